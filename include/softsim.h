@@ -118,11 +118,15 @@ typedef struct {
     int max_ls;               /* backtracking halvings cap */
     int tile_elems;           /* elements per tile (0 = library default) */
     int threads;              /* threads per element-kernel block (0 = default) */
-    int cg_kernel;            /* SIM_CG_AUTO: a whole CG solve in one kernel when
-                                 every tile of the mesh fits on the GPU at once (one
-                                 thread-block cluster for at most 16 tiles, else a
-                                 cooperative grid), else per-iteration kernels;
-                                 SIM_CG_ITERATION: always per-iteration kernels */
+    int cg_kernel;            /* SIM_CG_AUTO: a whole CG solve in one persistent
+                                 launch on the assembled edge blocks, with a two-level
+                                 preconditioner, when every CTA's part of the mesh fits
+                                 on the GPU at once (one CTA or thread-block cluster
+                                 for small meshes, else a cooperative grid; about
+                                 580,000 vertices in 3D), else per-iteration kernels;
+                                 SIM_CG_ITERATION: always per-iteration kernels,
+                                 matrix-free and without preconditioner.  The plan of
+                                 the persistent solver is built by the first solve */
 } sim_options;
 
 typedef struct {

@@ -42,8 +42,8 @@ class Simulator:
     include/softsim.h.  Host arrays (numpy or CPU tensors) are copied.
     ``tile_elems="auto"`` (or ``threads="auto"``) picks the tile shape with
     the autotuner (paper_2102_05791_gb300.autotune, cached per GPU).
-    ``cg_kernel="auto"`` runs each CG solve as one cooperative kernel when all
-    tiles fit on the GPU at once; ``"iteration"`` keeps per-iteration kernels.
+    ``cg_kernel="auto"`` runs each CG solve as one persistent, preconditioned
+    launch when the mesh fits it; ``"iteration"`` keeps per-iteration kernels.
     """
 
     def __init__(self, X, T, fixed=None, fiber=None, *, mu, lam, k_muscle=0.0, density=0.0, gravity=0.0,

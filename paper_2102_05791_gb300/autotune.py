@@ -3,8 +3,7 @@ batched persistent solver.
 
 For a mesh, tries candidate (elements per tile, threads per block) pairs:
 builds a handle for each, runs a short adjoint CG solve at the rest shape
-(48 iterations, in whichever way the handle runs CG: one cooperative kernel
-when all tiles fit on the GPU, else per-iteration kernels) and keeps the pair
+(48 iterations with the per-iteration kernels, whose tiles are what is tuned) and keeps the pair
 with the smallest time per CG iteration, measured with CUDA events around the
 solve.  Results are cached in a JSON file keyed by GPU name, dimension,
 element-count bucket (power of two) and precision, so later handles of a
@@ -23,8 +22,7 @@ import numpy as np
 
 CANDIDATES = {
     3: [(384, 128), (384, 256), (256, 128), (512, 128), (512, 256), (768, 256)],
-    # small tiles give small meshes more CTAs (a 4,096-triangle body has only 8 tiles of 512);
-    # at most 16 tiles run the CG solve as one thread-block cluster
+    # small tiles give small meshes more CTAs (a 4,096-triangle body has only 8 tiles of 512)
     2: [(512, 256), (512, 128), (384, 128), (768, 256), (1024, 256), (256, 256), (256, 128), (128, 128),
         (64, 64)],
 }
@@ -67,7 +65,7 @@ def measure(X, T, fixed, fiber, tile_elems: int, threads: int, precision: str = 
 
     from . import api
     sim = api.Simulator(X, T, fixed, fiber, precision=precision, tile_elems=tile_elems, threads=threads,
-                        max_adjoint_cg=iters, adjoint_rtol=1e-30, **material)
+                        max_adjoint_cg=iters, adjoint_rtol=1e-30, cg_kernel="iteration", **material)
     try:
         dev = sim.device
         x = sim.X

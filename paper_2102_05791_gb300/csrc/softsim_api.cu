@@ -13,8 +13,10 @@
 #include <cstdlib>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
+#include "cg_pcg.h"
 #include "internal.h"
 #include "softsim.h"
 #include "tiling.h"
@@ -59,6 +61,11 @@ struct sim_handle {
     void *vd = nullptr, *vr = nullptr, *vp = nullptr, *vAp = nullptr;  // CG vectors in the HVP precision
     double *work = nullptr, *lam = nullptr, *lacc = nullptr, *r64 = nullptr, *Hx = nullptr;
     int verbose = 0;
+    // persistent CG solver: its plan is built on the first CG solve, from the mesh kept until then
+    PcgDev pcg;
+    int pcg_state = 0;              // 0: not built, 1: usable, -1: the mesh does not fit it
+    std::vector<double> rest;
+    std::vector<int32_t> elems;
     double *rx[2] = {nullptr, nullptr}, *rv[2] = {nullptr, nullptr};  // rollout ping-pong
     DevScalars *sc = nullptr;
     DevScalars *sc_host = nullptr;  // pinned mirror
@@ -386,6 +393,10 @@ static int create_impl(sim_handle *h, const sim_mesh *mesh, const sim_material *
     c.vd.X = h->X;
     c.vd.mass = h->mass;
     c.vd.fixed = h->fixed;
+    if (h->opt.cg_kernel == SIM_CG_AUTO) {
+        h->rest.assign(mesh->rest_pos, mesh->rest_pos + nv * d);
+        h->elems.assign(mesh->elems, mesh->elems + ne * nc);
+    }
     TileDev &td = c.td;
     td.n_tiles = tb.n_tiles;
     td.max_te = tb.max_te;
@@ -677,6 +688,191 @@ static cudaGraphExec_t get_cg_while(sim_handle *h, const Phys &ph)
 // Rounds of the device-side loop that cover max_iter iterations, plus slack.
 static int cg_max_rounds(int max_iter) { return max_iter / kCgBody + 2; }
 
+// Parts (CTAs), aggregates and storage of the persistent CG solver for a mesh
+// of nv vertices.  The lines lie where both sides measured alike (microseconds
+// an iteration on GB300): one cluster exchanges in about 1 us, a grid in about
+// 2 us, so a cluster's 16 CTAs serve as long as their rows stay in shared
+// memory (3D FP32: 4.6 us at 1,260 vertices; 8.3 on a grid of 64 at 9,537, where
+// 16 CTAs need 18; 2D: 7.2 at 20,000).  FP64 arithmetic is scarce, so FP64
+// spreads over more CTAs earlier (16.0 us on 64 CTAs against 18.8 on 16 at 2,640
+// vertices).  More aggregates save iterations but cost a larger inverse (192
+// coarse unknowns: 0.12 ms, 96: 0.02 ms), which small meshes do not win back.
+// Rows beat colours until the part's rows no longer stay in L2 (3D FP32: 23.4
+// against 22.9 us at 122,000 vertices, 42.8 against 30.9 at 180,000).
+struct PcgSizes {
+    int n_cta, n_agg;
+    bool cluster, rows;
+};
+static PcgSizes pcg_sizes(int dim, bool f32, int64_t nv, int n_sm)
+{
+    const int nm = dim == 3 ? 6 : 3;
+    const int64_t per_cta = dim == 3 ? (f32 ? 270 : 100) : (f32 ? 1300 : 256);  // the most a cluster's CTA takes
+    int64_t g, a = std::max<int64_t>(1, std::min<int64_t>((nv <= 4096 ? kCgMaxCoarse / 2 : kCgMaxCoarse) / nm, nv / 18));
+    if (nv <= 16 * per_cta) {
+        g = f32 && nv <= 160 ? 1 : std::min<int64_t>(16, (nv + 31) / 32);
+        a = std::min(a, 16 * g);
+    } else {
+        g = std::min<int64_t>(n_sm, std::max<int64_t>(kCgMaxCoarse / nm, nv / (dim == 3 ? (f32 ? 150 : 40) : 256)));
+        a = std::min(a, g);
+        // aggregates of equally many parts (uneven ones cost a third more iterations at 9,537 vertices)
+        if (g / a * a * 10 < g * 9) a = g / ((g + a - 1) / a);
+        g = g / a * a;
+    }
+    if (a > g) a = a / g * g;
+    const int64_t per = (nv + g - 1) / g;
+    return {(int)g, (int)a, g > 1 && g <= 16, per <= (dim == 3 ? (f32 ? 750 : 600) : 2000)};
+}
+
+template <typename T>
+static int build_pcg(sim_handle *h)
+{
+    int n_sm = 0, rc;
+    CK(h, cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, h->device));
+    const PcgSizes z = pcg_sizes(h->dim, sizeof(T) == 4, h->nv, n_sm);
+    CgPlan P;
+    std::string err;
+    h->pcg_state = -1;
+    const bool ok = build_cg_plan(h->dim, h->nv, h->ne, h->rest.data(), h->elems.data(), h->tb.perm.data(), h->tb.ne_int,
+                                  z.n_cta, z.n_agg, z.rows, sizeof(T), z.n_cta > 1 && !z.cluster, P, err);
+    std::vector<double>().swap(h->rest);
+    std::vector<int32_t>().swap(h->elems);
+    if (!ok) {
+        if (h->verbose) fprintf(stderr, "[softsim] per-iteration CG kernels: %s\n", err.c_str());
+        return SIM_OK;
+    }
+    PcgDev &pd = h->pcg;
+    pd.n_cta = P.n_cta;
+    pd.n_agg = P.n_agg;
+    pd.n_modes = P.n_modes;
+    pd.n_coarse = P.n_agg * P.n_modes;
+    pd.ns = P.ns;
+    pd.max_halo = P.max_halo;
+    pd.max_entries = P.max_entries;
+    pd.max_chunks = P.max_chunks;
+    pd.tpr = P.tpr;
+    pd.n_meta = P.n_meta;
+    pd.max_items = P.max_items;
+    pd.n_items = (int)P.item_agg.size();
+    pd.cluster = z.cluster ? 1 : 0;
+    pd.n_edges = P.n_edges;
+    pd.n_contrib = P.n_contrib;
+    pd.n_entries = (int64_t)P.ent_idx.size();
+    pd.n_chunks = (int64_t)P.chunk_n.size();
+    pd.inv_len = (float)(1.0 / P.length);
+    pd.n_citems = (int)P.citem_kind.size();
+    pd.n_ctgts = (int)P.ctgt_i.size();
+    if (!pcg_configure<T>(h->ctx, pd)) {
+        if (h->verbose) fprintf(stderr, "[softsim] per-iteration CG kernels: a part does not fit in shared memory\n");
+        return SIM_OK;
+    }
+    // one allocation for the plan's tables and one for the buffers, filled in
+    // two passes (sizes, then pointers): forty separate ones cost milliseconds
+    const size_t dd = (size_t)h->dim * h->dim, slots = (size_t)P.n_cta * P.ns, N = pd.n_coarse;
+    std::vector<unsigned char> host;
+    size_t at = 0;
+    unsigned char *dev = nullptr;
+    auto table = [&](const auto &v, auto **dst) {
+        const size_t bytes = v.size() * sizeof(v[0]);
+        if (dev) {
+            if (bytes) memcpy(host.data() + at, v.data(), bytes);
+            *dst = reinterpret_cast<decltype(&v[0])>(dev + at);
+        }
+        at += (bytes + 255) / 256 * 256;
+    };
+    auto tables = [&]() {
+        at = 0;
+        table(P.slot_gid, &pd.slot_gid);
+        table(P.grp_agg, &pd.grp_agg);
+        table(P.nslot, &pd.nslot);
+        table(P.halo_ptr, &pd.halo_ptr);
+        table(P.halo_slot, &pd.halo_slot);
+        table(P.item_ptr, &pd.item_ptr);
+        table(P.item_agg, &pd.item_agg);
+        table(P.agg_item, &pd.agg_item);
+        table(P.agg_ref, &pd.agg_ref);
+        table(P.chunk_ptr, &pd.chunk_ptr);
+        table(P.chunk_ent, &pd.chunk_ent);
+        table(P.chunk_n, &pd.chunk_n);
+        table(P.row_step, &pd.row_step);
+        table(P.ent_idx, &pd.ent_idx);
+        table(P.ent_edge, &pd.ent_edge);
+        table(P.cpos, &pd.cpos);
+        table(P.edge_lo, &pd.edge_lo);
+        table(P.edge_hi, &pd.edge_hi);
+        table(P.edge_ptr, &pd.edge_ptr);
+        table(P.seg_edge, &pd.seg_edge);
+        table(P.citem_kind, &pd.citem_kind);
+        table(P.citem_begin, &pd.citem_begin);
+        table(P.citem_end, &pd.citem_end);
+        table(P.ctgt_ptr, &pd.ctgt_ptr);
+        table(P.ctgt_i, &pd.ctgt_i);
+        table(P.ctgt_j, &pd.ctgt_j);
+    };
+    auto buffer = [&](size_t bytes, auto **dst) {
+        if (dev) *dst = reinterpret_cast<std::remove_reference_t<decltype(*dst)>>(dev + at);
+        at += (bytes + 255) / 256 * 256;
+    };
+    auto buffers = [&]() {
+        at = 0;
+        buffer(sizeof(T) * dd * P.n_contrib, &pd.contrib);
+        buffer(sizeof(T) * dd * P.n_edges, &pd.blk);
+        buffer((4 + sizeof(T) * dd) * P.ent_idx.size(), &pd.slices);
+        buffer(sizeof(float4) * slots, &pd.pos4);
+        buffer(sizeof(T) * 2 * slots, &pd.diag2);
+        buffer(sizeof(T) * (h->dim == 3 ? 6 : 3) * slots, &pd.dinv);
+        buffer(sizeof(T) * 4 * slots, &pd.zr);
+        buffer(sizeof(float) * 36 * pd.n_citems, &pd.cpart);
+        buffer(sizeof(float) * N * N, &pd.E);
+        buffer(sizeof(float) * N * N, &pd.Einv);
+        buffer(sizeof(uint2) * 2 * kPcgWords * P.n_cta, &pd.words);
+        buffer(sizeof(double) * P.n_cta, &pd.part0);
+    };
+    tables();
+    const size_t table_bytes = at;
+    buffers();
+    const size_t buffer_bytes = at;
+    void *d0 = dalloc(h, table_bytes), *d1 = d0 ? dalloc(h, buffer_bytes) : nullptr;
+    if (!d1) {  // without the memory the per-iteration kernels, which need none, do the solve
+        if (d0) {
+            cudaFree(d0);
+            h->allocs.pop_back();
+        }
+        return SIM_OK;
+    }
+    host.resize(table_bytes);
+    dev = static_cast<unsigned char *>(d0);
+    tables();
+    CK(h, cudaMemcpy(d0, host.data(), table_bytes, cudaMemcpyHostToDevice));
+    dev = static_cast<unsigned char *>(d1);
+    buffers();
+    pd.has_diag = h->mat.dt > 0.0 || h->mat.k_contact > 0.0 ? 1 : 0;
+    if (h->verbose)
+        fprintf(stderr, "[softsim] persistent CG: %d CTAs%s x %d threads, %d slots, %d halo, %d coarse, %s, %d stages\n",
+                pd.n_cta, pd.cluster ? " (cluster)" : "", pd.threads, pd.ns, pd.max_halo, pd.n_coarse,
+                pd.tpr ? "rows" : "colours", pd.stages);
+    h->pcg_state = 1;
+    return SIM_OK;
+}
+
+// Whether this handle's CG solves run as one persistent launch; builds its plan on the first call.
+template <typename T>
+static int use_pcg(sim_handle *h, bool *use)
+{
+    *use = false;
+    if (h->opt.cg_kernel != SIM_CG_AUTO || h->timing) return SIM_OK;
+    if (h->pcg_state == 0) {
+        int rc = SIM_OK;
+        try {
+            rc = build_pcg<T>(h);
+        } catch (const std::exception &) {  // no host memory for the plan: per-iteration kernels
+            h->pcg_state = -1;
+        }
+        if (rc) return rc;
+    }
+    *use = h->pcg_state == 1;
+    return SIM_OK;
+}
+
 // Runs CG until the device raises `done`: one launch of the device-side loop
 // (a single host synchronisation), or, with in-solve kernel timing on or
 // without conditional graph nodes, replays of a kCgBlock-iteration graph with
@@ -686,11 +882,6 @@ template <typename T>
 static int run_cg(sim_handle *h, const Phys &ph, int max_iter, cudaStream_t s)
 {
     int rc;
-    if (!h->timing && h->opt.cg_kernel == SIM_CG_AUTO && cg_coop_fits<T>(h->ctx)) {
-        CK(h, launch_cg_coop<T>(h->ctx, ph, View<T>::u(h), (T *)h->vd, (T *)h->vr, (T *)h->vp, (T *)h->vAp,
-                                View<T>::hp(h), s));
-        return read_scalars(h, s);
-    }
     refresh_cg_u(h, s);
     if (!h->timing) {
         cudaGraphExec_t wexec = get_cg_while<T>(h, ph);
@@ -757,6 +948,8 @@ static int newton_impl(sim_handle *h, bool dyn, sim_solve_stats *st, cudaStream_
         if (st) *st = S;
         return S.status;
     }
+    bool pcg;
+    if ((rc = use_pcg<T>(h, &pcg))) return rc;
     const double eps = 2.220446049250313e-16;
     int it = 0;
     for (;; ++it) {
@@ -766,11 +959,15 @@ static int newton_impl(sim_handle *h, bool dyn, sim_solve_stats *st, cudaStream_
         }
         if (it >= h->opt.max_newton) break;
         const double eta = std::min(h->opt.newton_forcing, std::sqrt(gn / g0));
-        launch_cg_init<T>(c, h->g, -1.0, (T *)h->vd, (T *)h->vr, (T *)h->vp, eta, h->opt.max_cg,
-                          cg_max_rounds(h->opt.max_cg), s);
-        CKL(h);
-        if ((rc = run_cg<T>(h, ph, h->opt.max_cg, s))) return rc;
-        S.cg_iters_total += h->sc_host->iter;
+        if (pcg) {  // the coarse operator of the first step serves the whole solve
+            launch_pcg_assemble<T>(c, h->pcg, ph, View<T>::u(h), h->u, it == 0, s);
+            CK(h, launch_pcg<T>(c, h->pcg, h->g, -1.0, (T *)h->vd, eta, h->opt.max_cg, s));
+        } else {
+            launch_cg_init<T>(c, h->g, -1.0, (T *)h->vd, (T *)h->vr, (T *)h->vp, eta, h->opt.max_cg,
+                              cg_max_rounds(h->opt.max_cg), s);
+            CKL(h);
+            if ((rc = run_cg<T>(h, ph, h->opt.max_cg, s))) return rc;
+        }
         launch_dir_check<T>(c, h->g, (T *)h->vd, s);
         CKL(h);
         // line search: t = 1, then batches of halvings
@@ -793,6 +990,7 @@ static int newton_impl(sim_handle *h, bool dyn, sim_solve_stats *st, cudaStream_
             CKL(h);
             if ((rc = read_scalars(h, s))) return rc;
             const double gd = h->sc_host->gd;
+            if (j0 == 0) S.cg_iters_total += h->sc_host->iter;
             for (int j = 0; j < nt; ++j) {
                 const double Et = h->sc_host->E[j], St = h->sc_host->S[j];
                 const double slack = 64.0 * eps * std::max(Sabs, St);
@@ -872,6 +1070,8 @@ static int adjoint_impl(sim_handle *h, bool dyn, const double *b, double *lambda
         if (st) *st = S;
         return S.status;
     }
+    bool pcg;
+    if ((rc = use_pcg<T>(h, &pcg))) return rc;
     double rn = bn;
     const double target = h->opt.adjoint_rtol * bn;
     const double inner = is_mixed(h) ? std::max(h->opt.adjoint_rtol, 1e-4) : h->opt.adjoint_rtol;
@@ -882,19 +1082,24 @@ static int adjoint_impl(sim_handle *h, bool dyn, const double *b, double *lambda
             break;
         }
         if (budget <= 0) break;
-        launch_cg_init<T>(c, h->r64, 1.0, (T *)h->vd, (T *)h->vr, (T *)h->vp, std::max(inner, 0.5 * target / rn),
-                          budget, cg_max_rounds(budget), s);
-        CKL(h);
-        if ((rc = run_cg<T>(h, ph, budget, s))) return rc;
-        const int it = h->sc_host->iter;
-        const bool neg = h->sc_host->negcurv != 0;
-        S.cg_iters_total += it;
-        budget -= std::max(it, 1);
+        const double rtol = std::max(inner, 0.5 * target / rn);
+        if (pcg) {
+            if (pass == 0) launch_pcg_assemble<T>(c, h->pcg, ph, View<T>::u(h), h->u, true, s);
+            CK(h, launch_pcg<T>(c, h->pcg, h->r64, 1.0, (T *)h->vd, rtol, budget, s));
+        } else {
+            launch_cg_init<T>(c, h->r64, 1.0, (T *)h->vd, (T *)h->vr, (T *)h->vp, rtol, budget, cg_max_rounds(budget), s);
+            CKL(h);
+            if ((rc = run_cg<T>(h, ph, budget, s))) return rc;
+        }
         launch_accumulate<T>(c, h->lacc, (const T *)h->vd, s);
         launch_hvp<double>(c, ph, h->u, h->lacc, h->Hx, h->hp64, s);
         launch_residual(c, h->work, h->Hx, h->r64, s);
         CKL(h);
         if ((rc = read_scalars(h, s))) return rc;
+        const int it = h->sc_host->iter;
+        const bool neg = h->sc_host->negcurv != 0;
+        S.cg_iters_total += it;
+        budget -= std::max(it, 1);
         const double rn_new = std::sqrt(h->sc_host->gn2);
         if (h->verbose)
             fprintf(stderr, "[softsim] adjoint pass %d: cg %d, |r|/|b| %.3e -> %.3e%s\n", pass, it, rn / bn,

@@ -1,5 +1,4 @@
-// Device functions of the tiled HVP shared by the per-iteration tile kernel
-// (elem_kernels.cu) and the cooperative CG kernel (cg_coop.cu): one element's
+// Device functions of the tiled HVP (elem_kernels.cu): one element's
 // dP(dF) from its record, the corner-force stores, and one local vertex's
 // fixed-order corner sum with its per-vertex terms.
 #pragma once
@@ -74,7 +73,7 @@ __device__ __forceinline__ void gather_corners(const uint16_t *inc, uint32_t w, 
 // staged u and v of its vertices, evaluates G = W dP(dF) Dm^-T plus the
 // muscle term, adds v_e . (H_e v_e) to qsum (CG), and writes the element's
 // corner forces to out + corner_base(le) (out = rec overwrites the record in
-// place; a separate buffer of the same stride keeps the record).
+// place).
 template <typename T, int D, bool CG, bool SPRING, int RS>
 __device__ __forceinline__ void hvp_element(const T *rec, int le, uint32_t cword, const T *suv, const Phys &ph,
                                             T mu, T lam, T sel, T kk, T &qsum, T *out)
