@@ -150,6 +150,9 @@ bool build_cg_plan(int dim, int64_t nv, int64_t ne, const double *X, const int32
     P.n_cta = n_cta;
     P.n_modes = dim == 3 ? 6 : 3;
     const int nc = dim + 1, np = nc * (nc - 1) / 2;
+    // a cluster's CTAs write their items into each other's shared memory instead
+    // of summing them: every aggregate lies in one CTA there
+    if (!on_grid) n_agg = std::max(n_agg, n_cta);
     const int per = n_agg >= n_cta ? n_agg / n_cta : 1;  // aggregates per CTA
     n_agg = n_agg >= n_cta ? per * n_cta : n_agg;
     P.n_agg = n_agg;

@@ -177,6 +177,7 @@ int main(int argc, char **argv)
     // aggregates and the items of the coarse matrix
     for (int a = 0; a < P.n_agg; ++a) {
         REQ(P.agg_item[a] < P.agg_item[a + 1]);
+        REQ(want > 16 || P.agg_item[a + 1] - P.agg_item[a] == 1);  // a cluster does not sum items
         for (int q = P.agg_item[a]; q < P.agg_item[a + 1]; ++q) REQ(P.item_agg[q] == a);
     }
     std::vector<int> slots(P.slot_gid.size(), 0), edges(P.n_edges, 0);

@@ -23,7 +23,7 @@ def checker(tmp_path_factory):
 @pytest.mark.parametrize("rows", [0, 1])
 @pytest.mark.parametrize("shuffle", [0, 1])
 @pytest.mark.parametrize("dim,nx,ny,nz,n_cta,n_agg", [
-    (2, 1, 1, 0, 1, 1), (2, 16, 8, 0, 1, 8), (2, 19, 7, 0, 5, 8), (2, 64, 32, 0, 16, 64), (2, 120, 61, 0, 75, 25),
+    (2, 1, 1, 0, 1, 1), (2, 16, 8, 0, 1, 8), (2, 19, 7, 0, 5, 8), (2, 64, 32, 0, 16, 64), (2, 10, 2, 0, 2, 1), (2, 9, 4, 0, 4, 2), (2, 120, 61, 0, 75, 25),
     (3, 1, 1, 1, 1, 1), (3, 3, 4, 5, 2, 6), (3, 13, 9, 8, 16, 32), (3, 25, 13, 12, 31, 31), (3, 33, 17, 15, 150, 30)])
 def test_plan_invariants(checker, dim, nx, ny, nz, n_cta, n_agg, shuffle, rows):
     for elt in (4, 8):

@@ -31,7 +31,7 @@ def _problem(dims, split, shuffle):
 
 
 @pytest.mark.parametrize("dims,split,precision,shuffle", [
-    ((1, 1), 0, "mixed", False), ((3, 3), 0, "mixed", False), ((3, 3), 0, "fp64", False), ((20, 9), 0, "mixed", True),
+    ((1, 1), 0, "mixed", False), ((3, 3), 0, "mixed", False), ((3, 3), 0, "fp64", False), ((10, 2), 0, "fp64", False), ((20, 9), 0, "mixed", True),
     ((64, 41), 0, "mixed", False), ((64, 41), 0, "fp64", True), ((190, 121), 0, "mixed", False),
     ((1, 1, 1), 6, "mixed", False), ((1, 1, 1), 5, "fp64", False), ((7, 5, 3), 5, "mixed", False),
     ((13, 9, 8), 6, "mixed", True), ((12, 8, 9), 5, "fp64", False), ((24, 14, 13), 6, "mixed", False),
