@@ -300,12 +300,14 @@ int sim_tile_stats(const sim_handle *h, int *n_tiles, double *elems_per_tile,
  * Many independent meshes of uneven size (same dim; materials, ground
  * friction included, may differ only in mu and lambda), each rolled out for
  * n_steps backward-Euler steps (Eq. opt-be) and differentiated by backpropagation through time, in ONE
- * persistent kernel launch replayed from a captured CUDA graph.  Each CTA
- * takes the next mesh (largest first) and runs its whole forward rollout
- * (Newton-CG per step) and backward pass (refined adjoint CG and parameter
- * VJP per step, Eq. dLda-re-ordered) with block-level synchronisation only.
- * Mixed precision as SIM_PREC_MIXED.  Deterministic: a mesh is always
- * computed by one CTA with a fixed thread count and fixed-order sums. */
+ * persistent kernel launch.  Each CTA -- for the largest meshes of a batch
+ * that leaves SMs idle, each thread-block cluster of up to 16 CTAs -- takes
+ * the next mesh (largest first) and runs its whole forward rollout (Newton-CG
+ * per step) and backward pass (refined adjoint CG and parameter VJP per step,
+ * Eq. dLda-re-ordered) with block- or cluster-level synchronisation only.
+ * Mixed precision as SIM_PREC_MIXED.  Deterministic: the number of CTAs and
+ * threads of a mesh is fixed when the batch is created, its sums have a fixed
+ * order. */
 typedef struct sim_batch sim_batch;
 
 /* Meshes, materials (dt > 0) and options as for sim_create, HOST arrays,

@@ -39,8 +39,7 @@ struct PcgDev {
     void *zr = nullptr;              // [n_cta*ns][4 or 2] published D^-1 r
     float *cpart = nullptr;          // [n_citems][36]
     float *E = nullptr, *Einv = nullptr;  // [n_coarse][n_coarse]
-    uint2 *words = nullptr;          // [2][n_cta][kPcgWords] (value, tag) words of a grid's exchanges
-    double *part0 = nullptr;         // [n_cta] |b|^2
+    unsigned long long *words = nullptr;          // [2][n_cta][kPcgWords] (value, tag) words of a grid's exchanges
 };
 
 // The edge blocks at displacement u, the vertex terms and the rotation arms (every CG solve's
@@ -55,7 +54,7 @@ template <typename T>
 bool pcg_configure(const Ctx &c, PcgDev &pd);
 
 // Solves A d = sign * b (b in FP64, pinned entries ignored; d zero there) to |r| <= rtol |b| in one launch;
-// results in sc as from the per-iteration kernels.
+// sc->gn2 holds |b|^2; results in sc as from the per-iteration kernels.
 template <typename T>
 cudaError_t launch_pcg(const Ctx &c, const PcgDev &pd, const double *b, double sign, T *d, double rtol, int max_iter,
                        cudaStream_t s);

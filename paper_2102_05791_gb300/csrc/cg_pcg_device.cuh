@@ -1,0 +1,1020 @@
+// Device side of the preconditioned conjugate gradients on assembled edge
+// blocks: the solve of one CTA's part, shared by the persistent solver of one
+// mesh (cg_pcg_kernel.cuh) and the batched solver (batched_kernel.cuh).
+#pragma once
+
+#include <cstdint>
+
+#include "cg_pcg.h"
+#include "grid_sync.cuh"
+#include "reduce.cuh"
+#include "tma.cuh"
+
+namespace softsim {
+
+namespace {
+
+constexpr int kMaxWarps = 16;
+
+template <typename T, int D>
+struct Row;  // published vector row: D values in 8- or 16-byte units
+template <>
+struct Row<float, 3> {
+    static constexpr int N = 4;
+};
+template <>
+struct Row<float, 2> {
+    static constexpr int N = 2;
+};
+template <>
+struct Row<double, 3> {
+    static constexpr int N = 4;
+};
+template <>
+struct Row<double, 2> {
+    static constexpr int N = 2;
+};
+
+template <typename T, int D>
+__device__ __forceinline__ void put_row(T *z, const T v[D])
+{
+    if constexpr (sizeof(T) == 4 && D == 3) {
+        *reinterpret_cast<float4 *>(z) = make_float4(v[0], v[1], v[2], 0.0f);
+    } else if constexpr (sizeof(T) == 4) {
+        *reinterpret_cast<float2 *>(z) = make_float2(v[0], v[1]);
+    } else {
+        *reinterpret_cast<double2 *>(z) = make_double2(v[0], v[1]);
+        if constexpr (D == 3) z[2] = v[2];
+    }
+}
+
+template <typename T, int D>
+__device__ __forceinline__ void get_row(const T *z, T v[D])
+{
+    if constexpr (sizeof(T) == 4 && D == 3) {
+        const float4 a = __ldcg(reinterpret_cast<const float4 *>(z));
+        v[0] = a.x, v[1] = a.y, v[2] = a.z;
+    } else if constexpr (sizeof(T) == 4) {
+        const float2 a = __ldcg(reinterpret_cast<const float2 *>(z));
+        v[0] = a.x, v[1] = a.y;
+    } else {
+        const double2 a = __ldcg(reinterpret_cast<const double2 *>(z));
+        v[0] = a.x, v[1] = a.y;
+        if constexpr (D == 3) v[2] = __ldcg(z + 2);
+    }
+}
+
+// z += Z c at a vertex with arm R (c: the aggregate's coarse values)
+template <typename T, int D>
+__device__ __forceinline__ void prolong_add(float4 R, const float *c, T z[D])
+{
+    if constexpr (D == 3) {
+        z[0] += T(c[0] + c[4] * R.z - c[5] * R.y);
+        z[1] += T(c[1] + c[5] * R.x - c[3] * R.z);
+        z[2] += T(c[2] + c[3] * R.y - c[4] * R.x);
+    } else {
+        z[0] += T(c[0] - c[2] * R.y);
+        z[1] += T(c[1] + c[2] * R.x);
+    }
+}
+
+// acc += Z^T f
+template <int D>
+__device__ __forceinline__ void restrict_to(float4 R, const float f[D], float *acc)
+{
+#pragma unroll
+    for (int c = 0; c < D; ++c) acc[c] += f[c];
+    if constexpr (D == 3) {
+        acc[3] += R.y * f[2] - R.z * f[1];
+        acc[4] += R.z * f[0] - R.x * f[2];
+        acc[5] += R.x * f[1] - R.y * f[0];
+    } else {
+        acc[2] += R.x * f[1] - R.y * f[0];
+    }
+}
+
+template <typename V>
+__device__ __forceinline__ V warp_all(V v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Sums of eight values over a warp with nine shuffles: each step halves the
+// values a lane carries; lane l ends with the total of value (l >> 2) & 7.
+__device__ __forceinline__ float warp_sum8(const float v[8])
+{
+    const int lane = threadIdx.x & 31;
+    float a[4], b[2], c;
+    const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        a[i] = (h4 ? v[i + 4] : v[i]) + __shfl_xor_sync(0xffffffffu, h4 ? v[i] : v[i + 4], 16);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) b[i] = (h3 ? a[i + 2] : a[i]) + __shfl_xor_sync(0xffffffffu, h3 ? a[i] : a[i + 2], 8);
+    c = (h2 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, h2 ? b[0] : b[1], 4);
+    c += __shfl_xor_sync(0xffffffffu, c, 2);
+    return c + __shfl_xor_sync(0xffffffffu, c, 1);
+}
+
+// Inverse of the symmetric block S (xx, xy, yy | xx, xy, xz, yy, yz, zz); a
+// block that is not positive definite becomes a multiple of the identity.
+template <typename T, int D>
+__device__ __forceinline__ void invert_sym(const T *S, T *out)
+{
+    if constexpr (D == 2) {
+        const T det = S[0] * S[2] - S[1] * S[1];
+        if (S[0] > T(0) && det > T(1e-6) * S[0] * S[2]) {
+            const T i = T(1) / det;
+            out[0] = S[2] * i;
+            out[1] = -S[1] * i;
+            out[2] = S[0] * i;
+        } else {
+            const T t = fabs(S[0]) + fabs(S[2]), i = t > T(0) ? T(1) / t : T(0);
+            out[0] = out[2] = i;
+            out[1] = T(0);
+        }
+    } else {
+        const T a = S[3] * S[5] - S[4] * S[4], b = S[2] * S[4] - S[1] * S[5], c = S[1] * S[4] - S[2] * S[3];
+        const T det = S[0] * a + S[1] * b + S[2] * c, m = S[0] * S[3] - S[1] * S[1];
+        if (S[0] > T(0) && m > T(1e-6) * S[0] * S[3] && det > T(1e-6) * m * S[5]) {
+            const T i = T(1) / det;
+            out[0] = a * i;
+            out[1] = b * i;
+            out[2] = c * i;
+            out[3] = (S[0] * S[5] - S[2] * S[2]) * i;
+            out[4] = (S[1] * S[2] - S[0] * S[4]) * i;
+            out[5] = m * i;
+        } else {
+            const T t = fabs(S[0]) + fabs(S[3]) + fabs(S[5]), i = t > T(0) ? T(1) / t : T(0);
+            out[0] = out[3] = out[5] = i;
+            out[1] = out[2] = out[4] = T(0);
+        }
+    }
+}
+
+template <typename T, int D>
+__device__ __forceinline__ void sym_mul(const T *S, const T r[D], T z[D])
+{
+    if constexpr (D == 2) {
+        z[0] = S[0] * r[0] + S[1] * r[1];
+        z[1] = S[1] * r[0] + S[2] * r[1];
+    } else {
+        z[0] = S[0] * r[0] + S[1] * r[1] + S[2] * r[2];
+        z[1] = S[1] * r[0] + S[3] * r[1] + S[4] * r[2];
+        z[2] = S[2] * r[0] + S[4] * r[1] + S[5] * r[2];
+    }
+}
+
+// What a CTA's threads share in the edge passes.
+struct Slice {
+    unsigned char *base;             // the slice in shared memory, or the ring
+    const unsigned char *rest;       // rows: the steps that stay in global memory
+    const uint32_t *meta;            // shared-memory copy of the chunk sizes (colours) or step offsets (rows)
+    uint64_t *full, *empty;
+    int n_chunks, nthr, stages, ns;
+    uint32_t stage_bytes, n_ent, n_rest;
+    int tpr, polls0;                 // threads per row; poll limit of the very first wait
+    int stage;                       // position in the ring (every thread keeps its own copy)
+    uint32_t phase;
+    volatile int *bad;
+};
+
+__device__ __forceinline__ void csync(int nthr) { asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory"); }
+
+template <typename T, int D>
+__device__ __forceinline__ void load_entry(const unsigned char *base, int n, int k, uint32_t &w, T *M)
+{
+    w = reinterpret_cast<const uint32_t *>(base)[k];
+    const T *val = reinterpret_cast<const T *>(base + (size_t)n * 4);
+#pragma unroll
+    for (int q = 0; q < D * D; ++q) M[q] = val[q * n + k];
+}
+
+// One pass over the CTA's edges in colour order: f(target, source, block) for
+// every entry, colours separated by barriers.  Two chunks of a colour are
+// loaded before either is used.
+template <typename T, int D, typename F>
+__device__ __forceinline__ void colour_pass(Slice &sl, F f)
+{
+    constexpr int DD = D * D;
+    size_t off = 0;
+    for (int c = 0; c < sl.n_chunks;) {
+        const int k = threadIdx.x;
+        uint32_t w[2] = {kCgPadEntry, kCgPadEntry}, cn = 0;
+        T M[2][DD];
+        int took = 0;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            if (u == 1 && ((cn & kCgLastOfColour) || c + 1 >= sl.n_chunks)) break;
+            cn = sl.meta[c + u];
+            const int n = (int)(cn & ~kCgLastOfColour);
+            const unsigned char *base = sl.base + off;
+            bool ok = true;
+            const int st = sl.stage;
+            if (sl.stages) {
+                base = sl.base + (size_t)st * sl.stage_bytes;
+                ok = mbar_wait_bounded(sl.full + st, sl.phase, sl.polls0);
+                if (!ok) *sl.bad = 1;  // nothing of the chunk is touched
+                sl.polls0 = kWaitLimit;
+                if (++sl.stage == sl.stages) sl.stage = 0, sl.phase ^= 1u;
+            } else {
+                off += (size_t)n * (4 + DD * sizeof(T));
+            }
+            if (ok && k < n) load_entry<T, D>(base, n, k, w[u], M[u]);
+            if (sl.stages) {
+                __syncwarp();
+                if ((threadIdx.x & 31) == 0)
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(sl.empty + st)) : "memory");
+            }
+            ++took;
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+            if (w[u] != kCgPadEntry) f((int)(w[u] & 0xffff), (int)(w[u] >> 16), M[u]);
+        c += took;
+        if (cn & kCgLastOfColour) csync(sl.nthr);
+    }
+}
+
+// One pass over the CTA's rows: tpr threads a row, add(acc, row, source,
+// block) for its entries, done(row, acc) once with the row's sum of K values.
+// Steps that did not fit in shared memory come from L2, U at a time.
+template <typename T, int D, int K, int U, typename A, typename F>
+__device__ __forceinline__ void row_pass(const Slice &sl, A add, F done)
+{
+    constexpr int DD = D * D;
+    const int lane = threadIdx.x & 31, nw = sl.nthr >> 5, tpr = sl.tpr, n_vw = sl.ns * tpr >> 5;
+    const int sh = 31 - __clz(tpr);
+    const uint32_t *rest_at = sl.meta + n_vw + 1;
+    for (int vw = threadIdx.x >> 5; vw < n_vw; vw += nw) {
+        const int row = (vw * 32 + lane) >> sh;
+        T acc[K];
+#pragma unroll
+        for (int q = 0; q < K; ++q) acc[q] = T(0);
+        if (sl.n_rest) {
+            const uint32_t e1 = rest_at[vw + 1];
+            const uint32_t *idx = reinterpret_cast<const uint32_t *>(sl.rest);
+            const T *val = reinterpret_cast<const T *>(sl.rest + (size_t)sl.n_rest * 4);
+            for (uint32_t s = rest_at[vw]; s < e1; s += U) {
+                uint32_t w[U];
+                T M[U][DD];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const size_t e = (size_t)(s + u) * 32 + lane;
+                    w[u] = s + u < e1 ? __ldcg(idx + e) : 0u;
+#pragma unroll
+                    for (int q = 0; q < DD; ++q) M[u][q] = s + u < e1 ? __ldcg(val + (size_t)q * sl.n_rest + e) : T(0);
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) add(acc, row, (int)(w[u] >> 16), M[u]);
+            }
+        }
+        const uint32_t s1 = sl.meta[vw + 1];
+#pragma unroll 3
+        for (uint32_t s = sl.meta[vw]; s < s1; ++s) {
+            uint32_t w;
+            T M[DD];
+            load_entry<T, D>(sl.base, (int)sl.n_ent, (int)(s * 32 + lane), w, M);
+            add(acc, row, (int)(w >> 16), M);
+        }
+        for (int o = 1; o < tpr; o <<= 1)
+#pragma unroll
+            for (int q = 0; q < K; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+        if ((lane & (tpr - 1)) == 0) done(row, acc);
+    }
+}
+
+template <typename V>
+__device__ __forceinline__ void st_dsmem(void *local, uint32_t rank, V v)
+{
+    const uint32_t a = dsmem_addr(local, rank);
+    if constexpr (sizeof(V) == 4)
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+    else
+        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+
+// (value, tag) words of the grid's exchanges: 8-byte scalars, so that a reader
+// sees a value with its tag or neither.
+__device__ __forceinline__ void put_word(unsigned long long *p, uint32_t v, uint32_t tag)
+{
+    asm volatile("st.volatile.global.u64 [%0], %1;" ::"l"(p), "l"((unsigned long long)tag << 32 | v) : "memory");
+}
+// Two neighbouring words; each carries its own tag.
+__device__ __forceinline__ ulonglong2 load_words(const unsigned long long *p)
+{
+    ulonglong2 w;
+    asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(w.x), "=l"(w.y) : "l"(p) : "memory");
+    return w;
+}
+
+// Vertex vector in shared memory: 2D FP32 rows in one 8-byte access.
+template <typename T, int D>
+__device__ __forceinline__ void ld_vec(const T *p, int k, T v[D])
+{
+    if constexpr (sizeof(T) == 4 && D == 2) {
+        const float2 a = reinterpret_cast<const float2 *>(p)[k];
+        v[0] = a.x, v[1] = a.y;
+    } else {
+#pragma unroll
+        for (int c = 0; c < D; ++c) v[c] = p[k * D + c];
+    }
+}
+template <typename T, int D>
+__device__ __forceinline__ void st_vec(T *p, int k, const T v[D])
+{
+    if constexpr (sizeof(T) == 4 && D == 2) {
+        reinterpret_cast<float2 *>(p)[k] = make_float2(v[0], v[1]);
+    } else {
+#pragma unroll
+        for (int c = 0; c < D; ++c) p[k * D + c] = v[c];
+    }
+}
+
+// Tables of CTA cta that a solve reads from shared memory (the caller synchronises).
+template <int D, typename T, bool ROWS>
+__device__ __forceinline__ void pcg_tables(const PcgDev &pd, int cta, bool grid, unsigned char *smem)
+{
+    const PcgSmem L(D, sizeof(T), pd.ns, pd.max_halo, pd.max_items, pd.n_coarse, pd.n_meta, grid ? pd.n_cta : 0);
+    uint32_t *meta = reinterpret_cast<uint32_t *>(smem + L.meta);
+    int32_t *shalo = reinterpret_cast<int32_t *>(smem + L.halo);
+    const int h0 = pd.halo_ptr[cta], nh = pd.halo_ptr[cta + 1] - h0;
+    if constexpr (ROWS) {
+        for (int k = threadIdx.x; k < pd.n_meta; k += blockDim.x) meta[k] = pd.row_step[(size_t)cta * pd.n_meta + k];
+    } else {
+        const int c0 = pd.chunk_ptr[cta], nch = pd.chunk_ptr[cta + 1] - c0;
+        for (int k = threadIdx.x; k < nch; k += blockDim.x) meta[k] = pd.chunk_n[c0 + k];
+    }
+    for (int k = threadIdx.x; k < nh; k += blockDim.x) shalo[k] = pd.halo_slot[h0 + k];
+}
+
+// The slice of CTA cta (stored by rows when ROWS) whose shared part or ring starts at smem + L.ring.
+template <int D, typename T, bool ROWS>
+__device__ __forceinline__ Slice pcg_slice(const PcgDev &pd, int cta, bool grid, unsigned char *smem, int polls,
+                                           volatile int *bad)
+{
+    const PcgSmem L(D, sizeof(T), pd.ns, pd.max_halo, pd.max_items, pd.n_coarse, pd.n_meta, grid ? pd.n_cta : 0);
+    const size_t esz = 4 + D * D * sizeof(T);
+    const int c0 = pd.chunk_ptr[cta], nch = pd.chunk_ptr[cta + 1] - c0;
+    Slice sl;
+    sl.n_ent = (uint32_t)(pd.chunk_ent[c0 + (ROWS ? 1 : nch)] - pd.chunk_ent[c0]);
+    sl.n_rest = ROWS ? (uint32_t)(pd.chunk_ent[c0 + 2] - pd.chunk_ent[c0 + 1]) : 0u;
+    sl.base = smem + L.ring;
+    sl.rest = pd.slices + ((size_t)pd.chunk_ent[c0] + sl.n_ent) * esz;
+    sl.meta = reinterpret_cast<const uint32_t *>(smem + L.meta);
+    sl.full = reinterpret_cast<uint64_t *>(smem);
+    sl.empty = sl.full + kPcgMaxStages;
+    sl.n_chunks = nch;
+    sl.nthr = pd.threads;
+    sl.stages = ROWS ? 0 : pd.stages;
+    sl.ns = pd.nslot[cta];
+    sl.stage_bytes = (uint32_t)(kCgChunk * esz);
+    sl.tpr = pd.tpr;
+    sl.polls0 = polls;
+    sl.stage = 0;
+    sl.phase = 0;
+    sl.bad = bad;
+    return sl;
+}
+
+struct PcgResult {
+    int iter, neg, fail;
+    double rr;
+};
+
+// The solve itself, by the consumer threads of one CTA (number cta of pd.n_cta)
+// whose slice sl and tables (pcg_tables) are in place: x with A x = sign b to
+// |r| <= rtol |b| goes to dout.  ROWS: the slice is stored by rows (see
+// cg_plan.h), else by colours.  grid: the CTAs are a grid, else one cluster or
+// one CTA; nb2: |b|^2;
+// new_coarse: the coarse
+// inverse is not the one of the CTA's previous solve.
+template <typename T, int D, int VPT, bool ROWS>
+__device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int cta, bool grid, unsigned char *smem,
+                                             const double *b, double sign, double nb2, T *dout, double rtol,
+                                             int max_iter, bool new_coarse)
+{
+    constexpr int NM = D == 3 ? 6 : 3, ND = D == 3 ? 6 : 3, DD = D * D, RN = Row<T, D>::N;
+    constexpr int NI = (NM + 1) / 2;       // pairs of words that hold a CTA's items
+    constexpr bool F32 = sizeof(T) == 4;
+    constexpr bool KEEP_Z = VPT <= 2;  // D^-1 r stays in registers between the phases
+    constexpr int VB = VPT < 2 ? VPT : 2;  // slots whose loads are issued together
+    constexpr int PB = VPT < 4 ? 4 : 2;    // loads of an exchange in flight per thread
+    __shared__ float sred[kMaxWarps * VPT][8];  // per warp, or per group of 32 slots: restriction, two dots
+    __shared__ T sbc[3];
+    __shared__ T sdot[2][kMaxWarps];            // the dots of the FP64 solver
+    __shared__ T sdots[3][kMaxWarps];           // dots of the CTAs of a cluster (or of the only CTA)
+    __shared__ float scown[kMaxWarps][8];       // coarse values of this CTA's aggregates
+    __shared__ int sgrp[kMaxWarps + 1];         // first group of 32 slots of an item
+    __shared__ int sok;
+    const int G = pd.n_cta, nthr = sl.nthr, nw = nthr >> 5, tid = threadIdx.x;
+    const int lane = tid & 31, wrp = tid >> 5, N = pd.n_coarse;
+    const int ns = sl.ns, s0 = cta * pd.ns;
+    const int nh = pd.halo_ptr[cta + 1] - pd.halo_ptr[cta];
+    const int i0 = pd.item_ptr[cta], ni = pd.item_ptr[cta + 1] - i0, a0 = pd.item_agg[i0];
+    const bool one = ni == 1, solo = G == 1;
+    const PcgSmem L(D, sizeof(T), pd.ns, pd.max_halo, pd.max_items, N, pd.n_meta, grid ? G : 0);
+    T *sp = reinterpret_cast<T *>(smem + L.p), *sy = reinterpret_cast<T *>(smem + L.y);
+    float *sE = reinterpret_cast<float *>(smem + L.e), *sc_ = reinterpret_cast<float *>(smem + L.c);
+    // ss: restricted residual, two buffers (a cluster's CTAs write the next one while this one is read)
+    float *ss = reinterpret_cast<float *>(smem + L.s), *ss_next = ss + N, *st_ = reinterpret_cast<float *>(smem + L.t);
+    const int32_t *shalo = reinterpret_cast<const int32_t *>(smem + L.halo);
+    uint32_t *sword = reinterpret_cast<uint32_t *>(smem + L.word);  // [G][kPcgWords] of a grid's exchange
+    int fail = 0;
+    for (int k = tid; k < kMaxWarps * VPT * 8; k += nthr) (&sred[0][0])[k] = 0.0f;
+    for (int k = tid; k < ns / 32; k += nthr) {
+        const int it = pd.grp_agg[(s0 >> 5) + k] - a0;
+        if (k == 0 || pd.grp_agg[(s0 >> 5) + k - 1] - a0 != it) sgrp[it] = k;
+        if (k == ns / 32 - 1) sgrp[ni] = ns / 32;
+    }
+    if (tid == 0) sok = 1;
+
+    // --- diagonal blocks: minus the sums of the edge blocks, plus the vertex terms
+    // per-slot arrays, looked up in the plan where they are used: held in registers
+    // their addresses would cost the kernel a dozen
+    auto dg = [&](int k) { return static_cast<const T *>(pd.diag2) + 2 * (int64_t)(s0 + k); };
+    auto dinv = [&](int q, int k) { return static_cast<T *>(pd.dinv) + (int64_t)q * pd.n_cta * pd.ns + s0 + k; };
+    auto zr = [&](int slot) { return static_cast<T *>(pd.zr) + (int64_t)slot * RN; };
+    auto pos = [&](int k) { return pd.pos4[s0 + k]; };
+    auto gid = [&](int k) { return pd.slot_gid[s0 + k]; };
+    {
+        T *sd = sp;  // [ND][ns]: fits in p and y
+        auto sym = [](const T *M, T *S) {
+            if constexpr (D == 3) {
+                S[0] = M[0], S[1] = T(0.5) * (M[1] + M[3]), S[2] = T(0.5) * (M[2] + M[6]);
+                S[3] = M[4], S[4] = T(0.5) * (M[5] + M[7]), S[5] = M[8];
+            } else {
+                S[0] = M[0], S[1] = T(0.5) * (M[1] + M[2]), S[2] = M[3];
+            }
+        };
+        if constexpr (ROWS) {
+            row_pass<T, D, ND, 2>(
+                sl,
+                [&](T *acc, int, int, const T *M) {
+                    T S[ND];
+                    sym(M, S);
+#pragma unroll
+                    for (int q = 0; q < ND; ++q) acc[q] -= S[q];
+                },
+                [&](int row, const T *acc) {
+#pragma unroll
+                    for (int q = 0; q < ND; ++q) sd[q * ns + row] = acc[q];
+                });
+        } else {
+            for (int k = tid; k < ND * ns; k += nthr) sd[k] = T(0);
+            csync(nthr);
+            colour_pass<T, D>(sl, [&](int i, int j, const T *M) {
+                T S[ND];
+                sym(M, S);
+#pragma unroll
+                for (int q = 0; q < ND; ++q) sd[q * ns + i] -= S[q];
+                if (j < ns)
+#pragma unroll
+                    for (int q = 0; q < ND; ++q) sd[q * ns + j] -= S[q];
+            });
+        }
+        csync(nthr);
+        for (int k = tid; k < ns; k += nthr) {
+            T S[ND], o[ND];
+#pragma unroll
+            for (int q = 0; q < ND; ++q) S[q] = sd[q * ns + k];
+            const T dh = dg(k)[0], dy = dg(k)[1];
+            if constexpr (D == 3)
+                S[0] += dh, S[3] += dy, S[5] += dh;
+            else
+                S[0] += dh, S[2] += dy;
+            invert_sym<T, D>(S, o);
+#pragma unroll
+            for (int q = 0; q < ND; ++q) *dinv(q, k) = o[q];
+        }
+        csync(nthr);
+    }
+    for (int k = tid; k < (ns + nh) * D; k += nthr) sp[k] = T(0);
+    for (int k = tid; new_coarse && k < ni * NM * N; k += nthr) {  // this CTA's rows of E^-1, symmetrised
+        const int r = a0 * NM + k / N, n = k % N;
+        sE[k] = 0.5f * (pd.Einv[(size_t)r * N + n] + pd.Einv[(size_t)n * N + r]);
+    }
+
+    auto rhs = [&](int k, int c) {  // an unused or pinned slot has none
+        const int g = k < ns ? gid(k) : -1;
+        return g >= 0 && !(__float_as_int(pos(k).w) >> 30) ? sign * b[(int64_t)g * D + c] : 0.0;
+    };
+    // Per-slot reduction values v: NM restricted components, then up to two
+    // dots (FP32 solver).  A CTA of one aggregate sums its slots first.
+    auto put_sum = [&](int m, const float v[8]) {
+        const float t = warp_sum8(v);
+        if ((lane & 3) == 0) sred[one ? wrp : m * nw + wrp][lane >> 2] = t;
+    };
+    // The CTA's nd dots (after put_sum): valid in the lanes < nd of the last warp.
+    auto cta_dot = [&](int nd) -> T {
+        T v = T(0);
+        if constexpr (F32) {
+            const int q = 6 + (lane & 1), h = lane >> 1, ng = one ? nw : ns / 32;
+            for (int g = h; g < ng; g += 16) v += sred[g][q];
+#pragma unroll
+            for (int o = 16; o > 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        } else if (lane < nd) {
+            for (int w = 0; w < nw; ++w) v += sdot[lane][w];
+        }
+        return v;
+    };
+    // Exchange of the restricted vector (into dst) and of nd dots (slot base of
+    // sdots, or words of the grid); also of the coarse values with with_c.  buf
+    // and tag name the grid's words; fence orders the rows published before.
+    auto exchange = [&](int nd, const T *dots, float *dst, bool with_c, int base, int buf, uint32_t tag) -> bool {
+        if constexpr (!F32) {
+            for (int q = 0; q < nd; ++q) {
+                const T v = wrp * 32 < ns ? warp_all(dots[q]) : T(0);  // the FP64 pipe is the bottleneck: no sums of zeros
+                if (lane == 0) sdot[q][wrp] = v;
+            }
+        }
+        csync(nthr);
+        const int q = lane & 7, h = lane >> 3;
+        unsigned long long *mine = pd.words + ((size_t)buf * G + cta) * kPcgWords;
+        if (grid && with_c && wrp == 0) __threadfence();  // the CTA's rows before its words
+        for (int it = wrp; it < ni; it += nw) {
+            float v = 0.0f;
+            if (one) {
+#pragma unroll
+                for (int g = 0; g < kMaxWarps; g += 4) v += sred[g + h][q];  // rows of absent warps are zero
+            } else {
+                for (int g = sgrp[it] + h; g < sgrp[it + 1]; g += 4) v += sred[g][q];
+            }
+            v += __shfl_xor_sync(0xffffffffu, v, 8);
+            v += __shfl_xor_sync(0xffffffffu, v, 16);
+            if (grid) {  // one aggregate a CTA
+                if (h == 0 && q < 2 * NI) put_word(mine + q, __float_as_uint(v), tag);
+                if (with_c && h == 1 && q < 2 * NI) put_word(mine + 8 + q, q < NM ? __float_as_uint(scown[0][q]) : 0u, tag);
+            } else if (q < NM) {
+                const int n = (a0 + it) * NM + q;
+                const float c = with_c ? scown[it][q] : 0.0f;
+                if (solo) {
+                    dst[n] = v;
+                    if (with_c) sc_[n] = c;
+                } else {
+                    for (int k = h; k < G; k += 4) {
+                        st_dsmem(dst + n, (uint32_t)k, v);
+                        if (with_c) st_dsmem(sc_ + n, (uint32_t)k, c);
+                    }
+                }
+            }
+        }
+        if (nd > 0 && wrp == nw - 1) {
+            const T v = cta_dot(nd);
+            if (grid) {
+                if (lane < (F32 ? 2 : nd)) {
+                    if constexpr (F32) {
+                        put_word(mine + 14 + lane, __float_as_uint(v), tag);
+                    } else {
+                        put_word(mine + 14 + 2 * lane, (uint32_t)__double2loint(v), tag);
+                        put_word(mine + 15 + 2 * lane, (uint32_t)__double2hiint(v), tag);
+                    }
+                }
+            } else if (solo) {
+                if (lane < nd) sdots[base + lane][0] = v;
+            } else {
+                for (int d = 0; d < nd; ++d) {
+                    const T w = __shfl_sync(0xffffffffu, v, d);
+                    if (lane < G) st_dsmem(&sdots[base + d][cta], (uint32_t)lane, w);
+                }
+            }
+        }
+        if (solo) {
+            csync(nthr);
+            return true;
+        }
+        if (!grid) {
+            cluster_sync();
+            return true;
+        }
+        // the words of every CTA (items and dots) and, with_c, the coarse values of
+        // every aggregate's first CTA; PB loads in flight before the first is looked at
+        const unsigned long long *all = pd.words + (size_t)buf * G * kPcgWords;
+        const int nt = NI + (F32 ? (nd > 0) : nd), n_cta_load = G * nt, n_load = n_cta_load + (with_c ? pd.n_agg * NI : 0);
+        auto at = [&](int k) {
+            if (k >= n_cta_load) {
+                const int a = (k - n_cta_load) / NI;
+                return pd.agg_item[a] * kPcgWords + 8 + 2 * (k - n_cta_load - a * NI);
+            }
+            const int g = k / nt, j = k - g * nt;
+            return g * kPcgWords + 2 * (j < NI ? j : 7 + j - NI);
+        };
+        bool ok = true;
+        for (int k0 = tid; k0 < n_load; k0 += PB * nthr) {
+            ulonglong2 w[PB];
+            int o[PB];
+#pragma unroll
+            for (int u = 0; u < PB; ++u)
+                if (k0 + u * nthr < n_load) {
+                    o[u] = at(k0 + u * nthr);
+                    w[u] = load_words(all + o[u]);
+                }
+#pragma unroll
+            for (int u = 0; u < PB; ++u) {
+                if (k0 + u * nthr >= n_load) break;
+                for (int i = 0; ok && ((uint32_t)(w[u].x >> 32) != tag || (uint32_t)(w[u].y >> 32) != tag); ++i) {
+                    if (i >= kGridWaitPolls) ok = false;
+                    w[u] = load_words(all + o[u]);
+                }
+                sword[o[u]] = (uint32_t)w[u].x;
+                sword[o[u] + 1] = (uint32_t)w[u].y;
+            }
+        }
+        if (!ok) sok = 0;
+        if (with_c) __threadfence();  // the rows read next are those published before the words
+        csync(nthr);
+        for (int n = tid; n < N; n += nthr) {
+            const int a = n / NM, j = n - a * NM, g0 = pd.agg_item[a], g1 = pd.agg_item[a + 1];
+            float v = 0.0f;
+            for (int g = g0; g < g1; ++g) v += __uint_as_float(sword[g * kPcgWords + j]);
+            dst[n] = v;
+            if (with_c) sc_[n] = __uint_as_float(sword[g0 * kPcgWords + 8 + j]);
+        }
+        csync(nthr);
+        return sok != 0;
+    };
+    // This lane's share of dot d of the last exchange (every warp sums the CTAs alike).
+    auto dot_part = [&](int base, int d) -> T {
+        T v = T(0);
+        if (!grid) {
+            if (lane < G) v = sdots[base + d][lane];
+        } else {
+            for (int g = lane; g < G; g += 32) {
+                if constexpr (F32)
+                    v += __uint_as_float(sword[g * kPcgWords + 14 + d]);
+                else
+                    v += __hiloint2double((int)sword[g * kPcgWords + 15 + 2 * d], (int)sword[g * kPcgWords + 14 + 2 * d]);
+            }
+        }
+        return v;
+    };
+    auto swap_s = [&]() {
+        float *t = ss;
+        ss = ss_next;
+        ss_next = t;
+    };
+    auto coarse_part = [&]() -> T {  // Z^T r . c
+        float v = 0.0f;
+#pragma unroll
+        for (int u = 0; u < kCgMaxCoarse / 32; ++u) {
+            const int n = lane + 32 * u;
+            if (n < N) v = fmaf(ss[n], sc_[n], v);
+        }
+        return T(v);
+    };
+    // The coarse values of this CTA's aggregates from the restricted residual ss
+    // - alpha st_: a warp per row of E^-1, or, with more rows than warps, eight
+    // lanes per row.
+    auto coarse = [&](float alpha, bool with_t) {
+        if (ni * NM <= nw) {
+            if (wrp < ni * NM) {
+                float v = 0.0f;
+#pragma unroll
+                for (int u = 0; u < kCgMaxCoarse / 32; ++u) {
+                    const int n = lane + 32 * u;
+                    if (n < N) v = fmaf(sE[wrp * N + n], with_t ? fmaf(-alpha, st_[n], ss[n]) : ss[n], v);
+                }
+                v = warp_all(v);
+                if (lane == 0) scown[wrp / NM][wrp % NM] = v;
+            }
+        } else {
+            const int sub = lane & 7;
+            for (int row = wrp * 4 + (lane >> 3); row - (lane >> 3) < ni * NM; row += nw * 4) {
+                float v = 0.0f;
+                if (row < ni * NM)
+#pragma unroll 4
+                    for (int n = sub; n < N; n += 8)
+                        v = fmaf(sE[row * N + n], with_t ? fmaf(-alpha, st_[n], ss[n]) : ss[n], v);
+                v += __shfl_xor_sync(0xffffffffu, v, 1);
+                v += __shfl_xor_sync(0xffffffffu, v, 2);
+                v += __shfl_xor_sync(0xffffffffu, v, 4);
+                if (sub == 0 && row < ni * NM) scown[row / NM][row % NM] = v;
+            }
+        }
+    };
+
+    T x[VPT][D], r[VPT][D], zk[KEEP_Z ? VPT : 1][D];
+#pragma unroll
+    for (int m = 0; m < VPT; ++m)
+#pragma unroll
+        for (int c = 0; c < D; ++c) x[m][c] = T(0);
+    int it = 0, neg = 0;
+    T rr = T(1), rz = T(0);
+    const T tol2 = T(rtol * rtol);
+    bool run = !fail && nb2 > 0.0 && isfinite(nb2) && max_iter > 0 && rtol < 1.0;
+    if (*sl.bad) run = false, fail = 1;
+    // D^-1 r of slot k (S: its inverse diagonal block): publishes the row, adds to the reduction values
+    auto residual = [&](int m, int k, const T *S, float4 R, T *rm, float v[8], T &d_rr, T &d_rz) {
+        T z[D];
+        sym_mul<T, D>(S, rm, z);
+        put_row<T, D>(zr(s0 + k), z);
+        float f[D];
+#pragma unroll
+        for (int c = 0; c < D; ++c) {
+            if constexpr (KEEP_Z) zk[m][c] = z[c];
+            f[c] = (float)rm[c];
+            d_rr += rm[c] * rm[c];
+            d_rz += rm[c] * z[c];
+        }
+        restrict_to<D>(R, f, v);
+    };
+    uint32_t tag = 1;
+    if (run) {
+        const double scale = 1.0 / sqrt(nb2);
+        float v[8] = {};
+        T d_rr = T(0), d_rz = T(0);
+#pragma unroll
+        for (int m = 0; m < VPT; ++m) {
+            const int k = tid + m * nthr;
+#pragma unroll
+            for (int c = 0; c < D; ++c) r[m][c] = T(rhs(k, c) * scale);
+            if (k < ns) {
+                T S[ND];
+#pragma unroll
+                for (int q = 0; q < ND; ++q) S[q] = *dinv(q, k);
+                residual(m, k, S, pos(k), r[m], v, d_rr, d_rz);
+                if (!one) {
+                    put_sum(m, v);
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) v[q] = 0.0f;
+                }
+            }
+        }
+        if (one) put_sum(0, v);
+        if (!exchange(0, nullptr, ss, false, 0, 0, tag)) fail = 1;
+        coarse(0.0f, false);
+        // again with the coarse values and r.z
+        if constexpr (F32) {
+            const float t = warp_all((float)d_rz);
+            if (lane == 0) sred[wrp][6] = t;
+        }
+        if (!exchange(1, &d_rz, ss_next, true, 1, 1, tag)) fail = 1;
+        swap_s();
+        rz = warp_all(dot_part(1, 0) + coarse_part());
+    }
+    T beta = T(0);
+    while (run && !fail) {
+        ++tag;
+        // 1. p = z + beta p at own and halo vertices; A p
+#pragma unroll 2
+        for (int h = tid; h < nh; h += nthr) {
+            const int s = shalo[h];
+            T z[D], pv[D];
+            get_row<T, D>(zr(s), z);
+            const float4 R = pd.pos4[s];
+            const int w = __float_as_int(R.w);
+            ld_vec<T, D>(sp, ns + h, pv);
+            prolong_add<T, D>(R, sc_ + (w & 0xffff) * NM, z);
+#pragma unroll
+            for (int c = 0; c < D; ++c) pv[c] = (w >> 30) ? T(0) : z[c] + beta * pv[c];
+            st_vec<T, D>(sp, ns + h, pv);
+        }
+#pragma unroll
+        for (int m0 = 0; m0 < VPT; m0 += VB) {
+            T z[VB][D];
+            float4 R[VB];
+#pragma unroll
+            for (int u = 0; u < VB; ++u) {
+                const int k = tid + (m0 + u) * nthr;
+                if (k >= ns) continue;
+                R[u] = pos(k);
+                if constexpr (KEEP_Z) {
+#pragma unroll
+                    for (int c = 0; c < D; ++c) z[u][c] = zk[m0 + u][c];
+                } else {
+                    get_row<T, D>(zr(s0 + k), z[u]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < VB; ++u) {
+                const int k = tid + (m0 + u) * nthr;
+                if (k >= ns) continue;
+                const int w = __float_as_int(R[u].w);
+                T pv[D];
+                ld_vec<T, D>(sp, k, pv);
+                prolong_add<T, D>(R[u], sc_ + (w & 0xffff) * NM, z[u]);
+#pragma unroll
+                for (int c = 0; c < D; ++c) pv[c] = (w >> 30) ? T(0) : z[u][c] + beta * pv[c];
+                st_vec<T, D>(sp, k, pv);
+                if constexpr (!ROWS) {
+                    const T zero[D] = {};
+                    st_vec<T, D>(sy, k, zero);
+                }
+            }
+        }
+        csync(nthr);
+        if constexpr (ROWS) {
+            row_pass<T, D, D, (VPT == 1 ? 3 : 2)>(
+                sl,
+                [&](T *acc, int row, int j, const T *M) {
+                    T pi[D], d[D];
+                    ld_vec<T, D>(sp, row, pi);
+                    ld_vec<T, D>(sp, j, d);
+#pragma unroll
+                    for (int c = 0; c < D; ++c) d[c] -= pi[c];
+#pragma unroll
+                    for (int a = 0; a < D; ++a)
+#pragma unroll
+                        for (int c = 0; c < D; ++c) acc[a] += M[a * D + c] * d[c];
+                },
+                [&](int row, const T *acc) { st_vec<T, D>(sy, row, acc); });
+            csync(nthr);
+        } else {
+            colour_pass<T, D>(sl, [&](int i, int j, const T *M) {
+                T pi[D], d[D], y[D];
+                ld_vec<T, D>(sp, i, pi);
+                ld_vec<T, D>(sp, j, d);
+                ld_vec<T, D>(sy, i, y);
+#pragma unroll
+                for (int c = 0; c < D; ++c) d[c] -= pi[c];
+#pragma unroll
+                for (int a = 0; a < D; ++a)
+#pragma unroll
+                    for (int c = 0; c < D; ++c) y[a] += M[a * D + c] * d[c];
+                st_vec<T, D>(sy, i, y);
+                if (j < ns) {
+                    ld_vec<T, D>(sy, j, y);
+#pragma unroll
+                    for (int a = 0; a < D; ++a)
+#pragma unroll
+                        for (int c = 0; c < D; ++c) y[a] -= M[c * D + a] * d[c];
+                    st_vec<T, D>(sy, j, y);
+                }
+            });
+        }
+        {
+            float v[8] = {};
+            T dot = T(0);
+#pragma unroll
+            for (int m0 = 0; m0 < VPT; m0 += VB) {
+                float4 R[VB];
+                T dh[VB], dy[VB];
+#pragma unroll
+                for (int u = 0; u < VB; ++u) {
+                    const int k = tid + (m0 + u) * nthr;
+                    if (k >= ns) continue;
+                    R[u] = pos(k);
+                    dh[u] = dy[u] = T(0);
+                    if (pd.has_diag) dh[u] = dg(k)[0], dy[u] = dg(k)[1];
+                }
+#pragma unroll
+                for (int u = 0; u < VB; ++u) {
+                    const int k = tid + (m0 + u) * nthr;
+                    if (k >= ns) continue;
+                    float f[D];
+                    T pv[D], y[D];
+                    const bool fx = (__float_as_int(R[u].w) >> 30) != 0;
+                    ld_vec<T, D>(sp, k, pv);
+                    ld_vec<T, D>(sy, k, y);
+#pragma unroll
+                    for (int c = 0; c < D; ++c) {
+                        y[c] = fx ? T(0) : y[c] + (c == 1 ? dy[u] : dh[u]) * pv[c];
+                        f[c] = (float)y[c];
+                        dot += pv[c] * y[c];
+                    }
+                    st_vec<T, D>(sy, k, y);
+                    restrict_to<D>(R[u], f, v);
+                    if (!one) {
+                        if constexpr (F32) v[6] = (float)dot;
+                        put_sum(m0 + u, v);
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) v[q] = 0.0f;
+                        if constexpr (F32) dot = T(0);
+                    }
+                }
+            }
+            if (one) {
+                if constexpr (F32) v[6] = (float)dot;
+                put_sum(0, v);
+            }
+            if (*sl.bad) {  // a chunk never came: the others give up at their next wait
+                fail = 1;
+                break;
+            }
+            if (!exchange(1, &dot, st_, false, 0, 0, tag)) {
+                fail = 1;
+                break;
+            }
+        }
+        // 2. alpha; x, r, D^-1 r; the coarse values; r.r and r.z
+        T pAp, alpha;
+        if constexpr (F32) {
+            pAp = solo ? sdots[0][0] : warp_all(dot_part(0, 0));
+            alpha = __fdividef(rz, pAp);
+        } else {  // one warp forms the FP64 scalars
+            if (wrp == 0) {
+                pAp = warp_all(dot_part(0, 0));
+                if (lane == 0) {
+                    sbc[0] = pAp;
+                    sbc[1] = rz / pAp;
+                }
+            }
+            csync(nthr);
+            pAp = sbc[0];
+            alpha = sbc[1];
+        }
+        if (!(pAp > T(0)) || !isfinite(pAp)) {
+            neg = 1;
+            if (it == 0)  // the preconditioned steepest-descent direction
+#pragma unroll
+                for (int m = 0; m < VPT; ++m)
+#pragma unroll
+                    for (int c = 0; c < D; ++c)
+                        if (tid + m * nthr < ns) x[m][c] = sp[(tid + m * nthr) * D + c];
+            break;
+        }
+        coarse((float)alpha, true);
+        {
+            float v[8] = {};
+            T dots[2] = {T(0), T(0)};
+#pragma unroll
+            for (int m0 = 0; m0 < VPT; m0 += VB) {
+                T S[VB][ND];
+                float4 R[VB];
+#pragma unroll
+                for (int u = 0; u < VB; ++u) {
+                    const int k = tid + (m0 + u) * nthr;
+                    if (k >= ns) continue;
+                    R[u] = pos(k);
+#pragma unroll
+                    for (int q = 0; q < ND; ++q) S[u][q] = *dinv(q, k);
+                }
+#pragma unroll
+                for (int u = 0; u < VB; ++u) {
+                    const int m = m0 + u, k = tid + m * nthr;
+                    if (k >= ns) continue;
+                    T pv[D], y[D];
+                    ld_vec<T, D>(sp, k, pv);
+                    ld_vec<T, D>(sy, k, y);
+#pragma unroll
+                    for (int c = 0; c < D; ++c) {
+                        x[m][c] += alpha * pv[c];
+                        r[m][c] -= alpha * y[c];
+                    }
+                    residual(m, k, S[u], R[u], r[m], v, dots[0], dots[1]);
+                    if (!one) {
+                        if constexpr (F32) v[6] = (float)dots[0], v[7] = (float)dots[1];
+                        put_sum(m, v);
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) v[q] = 0.0f;
+                        if constexpr (F32) dots[0] = dots[1] = T(0);
+                    }
+                }
+            }
+            if (one) {
+                if constexpr (F32) v[6] = (float)dots[0], v[7] = (float)dots[1];
+                put_sum(0, v);
+            }
+            if (!exchange(2, dots, ss_next, true, 1, 1, tag)) {
+                fail = 1;
+                break;
+            }
+            swap_s();
+        }
+        ++it;
+        T rz_new;
+        if (F32 || wrp == 0) {
+            rr = dot_part(1, 0);
+            rz_new = dot_part(1, 1) + coarse_part();
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                rr += __shfl_xor_sync(0xffffffffu, rr, o);
+                rz_new += __shfl_xor_sync(0xffffffffu, rz_new, o);
+            }
+        }
+        if constexpr (F32) {
+            beta = __fdividef(rz_new, rz);
+        } else {
+            if (wrp == 0 && lane == 0) {
+                sbc[0] = rr;
+                sbc[1] = rz_new;
+                sbc[2] = rz_new / rz;
+            }
+            csync(nthr);
+            rr = sbc[0];
+            rz_new = sbc[1];
+            beta = sbc[2];
+        }
+        rz = rz_new;
+        if (!(rr > tol2) || it >= max_iter || !isfinite(rr) || !(rz > T(0))) break;
+    }
+    const double bnorm = nb2 > 0.0 && isfinite(nb2) ? sqrt(nb2) : 0.0;
+#pragma unroll
+    for (int m = 0; m < VPT; ++m) {
+        const int k = tid + m * nthr;
+        if (k >= ns || gid(k) < 0) continue;
+#pragma unroll
+        for (int c = 0; c < D; ++c) dout[(int64_t)gid(k) * D + c] = T((double)x[m][c] * bnorm);
+    }
+    PcgResult res;
+    res.iter = it;
+    res.neg = neg;
+    res.fail = fail;
+    res.rr = (double)rr * bnorm * bnorm;
+    return res;
+}
+
+}  // namespace
+}  // namespace softsim

@@ -3,54 +3,21 @@
 
 #include <algorithm>
 #include <array>
-#include <atomic>
 #include <cmath>
-#include <new>
 #include <numeric>
-#include <system_error>
-#include <thread>
+
+#include "host_parallel.h"
 
 namespace softsim {
 
-// f(i) for i in [0, n), the indices handed out in blocks to a few threads
-// (every f writes its own outputs only).  What an f throws is thrown again here.
-// work_size: vertices behind all of it (1-2 us of work each); a thread costs tens
-// of microseconds to start, so it is given at least 512 of them.
-template <typename F>
-static void parallel_for(int64_t work_size, int64_t n, int64_t block, F f)
+// Recursive coordinate bisection: orders ids so that unit k, of weight
+// w[k + 1] - w[k], is ids[cut[first + k]] .. ids[cut[first + k + 1]) with its
+// share of the n ids; the longest axis is cut at the quantile of half the units.
+static void bisect(int dim, const double *X, int32_t *ids, int64_t n, const int *w, int n_units, int64_t base,
+                   int64_t *cut, int depth)
 {
-    const int64_t n_blocks = (n + block - 1) / block;
-    const int n_thr = (int)std::min<int64_t>(
-        {n_blocks, work_size / 512 + 1, (int64_t)std::max(1u, std::thread::hardware_concurrency()), 16});
-    std::atomic<int64_t> next(0);
-    std::atomic<bool> failed(false);
-    auto work = [&]() {
-        try {
-            for (int64_t b; !failed && (b = next.fetch_add(1)) < n_blocks;)
-                for (int64_t i = b * block; i < std::min(n, (b + 1) * block); ++i) f(i);
-        } catch (...) {
-            failed = true;
-        }
-    };
-    std::vector<std::thread> th;
-    th.reserve(n_thr);
-    try {
-        for (int t = 1; t < n_thr; ++t) th.emplace_back(work);
-    } catch (const std::system_error &) {  // fewer threads do
-    }
-    work();
-    for (auto &t : th) t.join();
-    if (failed) throw std::bad_alloc();
-}
-
-// Recursive coordinate bisection: orders ids so that part k of n_parts is
-// ids[cut[k]] .. ids[cut[k+1]) (sizes differ by at most one per level); the
-// longest axis of the part is cut at its proportional quantile.
-static void bisect(int dim, const double *X, int32_t *ids, int64_t n, int n_parts, int first, int64_t base,
-                   std::vector<int64_t> &cut, int depth)
-{
-    if (n_parts == 1) {
-        cut[first] = base;
+    if (n_units == 1) {
+        cut[0] = base;
         return;
     }
     double lo[3], hi[3];
@@ -64,8 +31,8 @@ static void bisect(int dim, const double *X, int32_t *ids, int64_t n, int n_part
     int ax = 0;
     for (int c = 1; c < dim; ++c)
         if (hi[c] - lo[c] > hi[ax] - lo[ax]) ax = c;
-    const int left = n_parts / 2;
-    const int64_t m = n * left / n_parts;
+    const int left = n_units / 2;
+    const int64_t m = n * (w[left] - w[0]) / (w[n_units] - w[0]);
     std::nth_element(ids, ids + m, ids + n, [&](int32_t a, int32_t b) {
         const double xa = X[(int64_t)a * dim + ax], xb = X[(int64_t)b * dim + ax];
         return xa != xb ? xa < xb : a < b;
@@ -73,17 +40,14 @@ static void bisect(int dim, const double *X, int32_t *ids, int64_t n, int n_part
     std::thread t;
     if (depth > 0 && n > 20000) {
         try {
-            t = std::thread([&]() { bisect(dim, X, ids, m, left, first, base, cut, depth - 1); });
+            t = std::thread([&]() { bisect(dim, X, ids, m, w, left, base, cut, depth - 1); });
         } catch (const std::system_error &) {  // this thread does both halves
         }
     }
-    if (t.joinable()) {
-        bisect(dim, X, ids + m, n - m, n_parts - left, first + left, base + m, cut, depth - 1);
-        t.join();
-    } else {
-        bisect(dim, X, ids, m, left, first, base, cut, 0);
-        bisect(dim, X, ids + m, n - m, n_parts - left, first + left, base + m, cut, 0);
-    }
+    const bool both = !t.joinable();
+    if (both) bisect(dim, X, ids, m, w, left, base, cut, 0);
+    bisect(dim, X, ids + m, n - m, w + left, n_units - left, base + m, cut + left, both ? 0 : depth - 1);
+    if (!both) t.join();
 }
 
 // Position along a Morton curve through the box lo .. lo + ext (10 bits an axis).
@@ -142,6 +106,21 @@ struct CtaBuild {
 };
 }  // namespace
 
+int aggregates_per_part(int64_t v, int most, int threads)
+{
+    int best = 1;
+    int64_t best_slots = INT64_MAX;
+    for (int a = std::max(1, most); a >= 1; --a) {
+        const int64_t slots = a * (((v + a - 1) / a + 31) / 32 * 32);
+        if (slots <= threads || slots * 5 <= v * 6) return a;
+        if (slots < best_slots) {
+            best_slots = slots;
+            best = a;
+        }
+    }
+    return best;
+}
+
 bool build_cg_plan(int dim, int64_t nv, int64_t ne, const double *X, const int32_t *T, const int32_t *perm,
                    int64_t ne_int, int n_cta, int n_agg, bool rows, int elt, bool on_grid, CgPlan &P, std::string &err)
 {
@@ -166,8 +145,21 @@ bool build_cg_plan(int dim, int64_t nv, int64_t ne, const double *X, const int32
     std::vector<int32_t> ids(nv);
     std::iota(ids.begin(), ids.end(), 0);
     std::vector<int64_t> cut(n_parts + 1, 0);
-    bisect(dim, X, ids.data(), nv, n_parts, 0, 0, cut, 4);
-    cut[n_parts] = nv;
+    {
+        // the coarser level first (aggregates of one or more CTAs, or CTAs of one or
+        // more aggregates), so that both are compact
+        const int n_top = per > 1 ? n_cta : n_agg;
+        std::vector<int> w(n_top + 1), one(n_parts + 1);
+        for (int k = 0; k <= n_top; ++k) w[k] = (int)((int64_t)k * n_parts / n_top);
+        std::iota(one.begin(), one.end(), 0);
+        std::vector<int64_t> top(n_top + 1, nv);
+        bisect(dim, X, ids.data(), nv, w.data(), n_top, 0, top.data(), 4);
+        parallel_for(nv, n_top, 1, [&](int64_t k) {
+            bisect(dim, X, ids.data() + top[k], top[k + 1] - top[k], one.data() + w[k], w[k + 1] - w[k], top[k],
+                   cut.data() + w[k], 0);
+        });
+        cut[n_parts] = nv;
+    }
     double lo[3], hi[3];
     for (int c = 0; c < dim; ++c) lo[c] = INFINITY, hi[c] = -INFINITY;
     for (int64_t i = 0; i < nv; ++i)
@@ -212,7 +204,11 @@ bool build_cg_plan(int dim, int64_t nv, int64_t ne, const double *X, const int32
     P.item_ptr.push_back(0);
     for (int c = 0; c < n_cta; ++c) {
         int s = 0;
-        const int last_agg = per > 1 ? (c + 1) * per - 1 : (int)((int64_t)c * n_agg / n_cta);
+        int last_agg = (c + 1) * per - 1;
+        if (per == 1) {  // the aggregate k whose parts k n_cta / n_agg .. hold part c
+            last_agg = (int)((int64_t)c * n_agg / n_cta);
+            while ((int64_t)(last_agg + 1) * n_cta / n_agg <= c) ++last_agg;
+        }
         for (int g = 0; g < ns / 32; ++g) P.grp_agg[(size_t)c * ns / 32 + g] = last_agg;
         for (int a = 0; a < per; ++a) {
             const int part = c * per + a, agg = per > 1 ? part : last_agg;

@@ -30,8 +30,8 @@
 // are ordered so that a warp's sources mostly lie in distinct banks.
 //
 // Aggregates (coarse space: the rigid motions of each) are unions of
-// contiguous slot ranges in part order: several per part on small meshes,
-// several parts per aggregate on large ones.
+// contiguous slot ranges in part order: one or several per part on small
+// meshes (always on a cluster), several parts per aggregate on large ones.
 #pragma once
 
 #include <cstdint>
@@ -46,7 +46,7 @@ constexpr uint32_t kCgLastOfColour = 0x80000000u;
 constexpr uint32_t kCgTransposed = 0x80000000u;
 constexpr int kPcgMaxStages = 8;
 constexpr int kPcgSmem = 226 * 1024;     // shared memory of one CTA, static part included
-constexpr int kPcgStatic = 6 * 1024;     // room for the kernels' static part when a slice is sized
+constexpr int kPcgStatic = 10 * 1024;     // room for the kernels' static part when a slice is sized
 constexpr int kPcgWords = 18;            // words of a CTA in a grid's exchange: items from 0, coarse values from 8, dots from 14
 constexpr int kCgMaxCoarse = 192;  // coarse unknowns (cg_assemble.cu inverts the coarse matrix in one CTA's registers)
 constexpr int kCgCoarseItem = 1024;  // edges or slots per partial sum of the coarse matrix
@@ -105,6 +105,12 @@ struct CgPlan {
     std::vector<int32_t> ctgt_ptr, ctgt_i, ctgt_j;
     double length = 1.0;               // scale of the rotation modes
 };
+
+// Aggregates per CTA, at most `most`, for parts of v vertices: the slots of an
+// aggregate are padded to a multiple of 32, so the largest number is taken that
+// keeps to `threads` slots (one a thread) or wastes less than a fifth of the
+// slots, else the least wasteful.
+int aggregates_per_part(int64_t v, int most, int threads);
 
 // rows: store the parts by rows; elt: bytes of a value of the solver; on_grid: the
 // CTAs are not one cluster.  perm: tile order -> caller order (-1 padding), ne_int entries; max_entries of any CTA

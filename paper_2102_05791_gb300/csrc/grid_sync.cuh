@@ -18,6 +18,14 @@ __device__ __forceinline__ void cluster_sync()
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// This CTA's rank in its cluster.
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
 // Address of the same shared-memory object in the CTA of the given cluster rank.
 __device__ __forceinline__ uint32_t dsmem_addr(const void *local, uint32_t rank)
 {

@@ -130,7 +130,6 @@ struct DevScalars {
     float alpha_f, beta_f;  // FP32 copies of alpha and beta for the FP32 vector kernels
     int iter, max_iter, done, negcurv;
     int cg_rounds, cg_max_rounds;  // body rounds of the device-side CG loop and their cap
-    unsigned int gs_count, gs_pad;  // grid-barrier word of the persistent CG kernel (zeroed before each launch)
     // Newton
     double gn2;      // |g|^2 of the FP64 gradient
     double gd;       // g . d

@@ -13,10 +13,10 @@
 #include <cstdlib>
 #include <cstring>
 #include <string>
-#include <type_traits>
 #include <vector>
 
 #include "cg_pcg.h"
+#include "cg_pcg_host.h"
 #include "internal.h"
 #include "softsim.h"
 #include "tiling.h"
@@ -714,12 +714,9 @@ static PcgSizes pcg_sizes(int dim, bool f32, int64_t nv, int n_sm)
     } else {
         g = std::min<int64_t>(n_sm, std::max<int64_t>(kCgMaxCoarse / nm, nv / (dim == 3 ? (f32 ? 150 : 40) : 256)));
         a = std::min(a, g);
-        // aggregates of equally many parts (uneven ones cost a third more iterations at 9,537 vertices)
-        if (g / a * a * 10 < g * 9) a = g / ((g + a - 1) / a);
-        g = g / a * a;
     }
-    if (a > g) a = a / g * g;
     const int64_t per = (nv + g - 1) / g;
+    if (a > g) a = g * aggregates_per_part(per, (int)(a / g), 512);
     return {(int)g, (int)a, g > 1 && g <= 16, per <= (dim == 3 ? (f32 ? 750 : 600) : 2000)};
 }
 
@@ -741,96 +738,14 @@ static int build_pcg(sim_handle *h)
         return SIM_OK;
     }
     PcgDev &pd = h->pcg;
-    pd.n_cta = P.n_cta;
-    pd.n_agg = P.n_agg;
-    pd.n_modes = P.n_modes;
-    pd.n_coarse = P.n_agg * P.n_modes;
-    pd.ns = P.ns;
-    pd.max_halo = P.max_halo;
-    pd.max_entries = P.max_entries;
-    pd.max_chunks = P.max_chunks;
-    pd.tpr = P.tpr;
-    pd.n_meta = P.n_meta;
-    pd.max_items = P.max_items;
-    pd.n_items = (int)P.item_agg.size();
-    pd.cluster = z.cluster ? 1 : 0;
-    pd.n_edges = P.n_edges;
-    pd.n_contrib = P.n_contrib;
-    pd.n_entries = (int64_t)P.ent_idx.size();
-    pd.n_chunks = (int64_t)P.chunk_n.size();
-    pd.inv_len = (float)(1.0 / P.length);
-    pd.n_citems = (int)P.citem_kind.size();
-    pd.n_ctgts = (int)P.ctgt_i.size();
+    pcg_sizes_of(P, z.cluster, h->mat.dt > 0.0 || h->mat.k_contact > 0.0, pd);
     if (!pcg_configure<T>(h->ctx, pd)) {
         if (h->verbose) fprintf(stderr, "[softsim] per-iteration CG kernels: a part does not fit in shared memory\n");
         return SIM_OK;
     }
-    // one allocation for the plan's tables and one for the buffers, filled in
-    // two passes (sizes, then pointers): forty separate ones cost milliseconds
-    const size_t dd = (size_t)h->dim * h->dim, slots = (size_t)P.n_cta * P.ns, N = pd.n_coarse;
-    std::vector<unsigned char> host;
-    size_t at = 0;
-    unsigned char *dev = nullptr;
-    auto table = [&](const auto &v, auto **dst) {
-        const size_t bytes = v.size() * sizeof(v[0]);
-        if (dev) {
-            if (bytes) memcpy(host.data() + at, v.data(), bytes);
-            *dst = reinterpret_cast<decltype(&v[0])>(dev + at);
-        }
-        at += (bytes + 255) / 256 * 256;
-    };
-    auto tables = [&]() {
-        at = 0;
-        table(P.slot_gid, &pd.slot_gid);
-        table(P.grp_agg, &pd.grp_agg);
-        table(P.nslot, &pd.nslot);
-        table(P.halo_ptr, &pd.halo_ptr);
-        table(P.halo_slot, &pd.halo_slot);
-        table(P.item_ptr, &pd.item_ptr);
-        table(P.item_agg, &pd.item_agg);
-        table(P.agg_item, &pd.agg_item);
-        table(P.agg_ref, &pd.agg_ref);
-        table(P.chunk_ptr, &pd.chunk_ptr);
-        table(P.chunk_ent, &pd.chunk_ent);
-        table(P.chunk_n, &pd.chunk_n);
-        table(P.row_step, &pd.row_step);
-        table(P.ent_idx, &pd.ent_idx);
-        table(P.ent_edge, &pd.ent_edge);
-        table(P.cpos, &pd.cpos);
-        table(P.edge_lo, &pd.edge_lo);
-        table(P.edge_hi, &pd.edge_hi);
-        table(P.edge_ptr, &pd.edge_ptr);
-        table(P.seg_edge, &pd.seg_edge);
-        table(P.citem_kind, &pd.citem_kind);
-        table(P.citem_begin, &pd.citem_begin);
-        table(P.citem_end, &pd.citem_end);
-        table(P.ctgt_ptr, &pd.ctgt_ptr);
-        table(P.ctgt_i, &pd.ctgt_i);
-        table(P.ctgt_j, &pd.ctgt_j);
-    };
-    auto buffer = [&](size_t bytes, auto **dst) {
-        if (dev) *dst = reinterpret_cast<std::remove_reference_t<decltype(*dst)>>(dev + at);
-        at += (bytes + 255) / 256 * 256;
-    };
-    auto buffers = [&]() {
-        at = 0;
-        buffer(sizeof(T) * dd * P.n_contrib, &pd.contrib);
-        buffer(sizeof(T) * dd * P.n_edges, &pd.blk);
-        buffer((4 + sizeof(T) * dd) * P.ent_idx.size(), &pd.slices);
-        buffer(sizeof(float4) * slots, &pd.pos4);
-        buffer(sizeof(T) * 2 * slots, &pd.diag2);
-        buffer(sizeof(T) * (h->dim == 3 ? 6 : 3) * slots, &pd.dinv);
-        buffer(sizeof(T) * 4 * slots, &pd.zr);
-        buffer(sizeof(float) * 36 * pd.n_citems, &pd.cpart);
-        buffer(sizeof(float) * N * N, &pd.E);
-        buffer(sizeof(float) * N * N, &pd.Einv);
-        buffer(sizeof(uint2) * 2 * kPcgWords * P.n_cta, &pd.words);
-        buffer(sizeof(double) * P.n_cta, &pd.part0);
-    };
-    tables();
-    const size_t table_bytes = at;
-    buffers();
-    const size_t buffer_bytes = at;
+    // one allocation for the plan's tables and one for the buffers: forty separate ones cost milliseconds
+    const size_t table_bytes = pcg_place_tables(P, pd, nullptr, nullptr, 0);
+    const size_t buffer_bytes = pcg_place_buffers<T>(P, pd, nullptr, 0);
     void *d0 = dalloc(h, table_bytes), *d1 = d0 ? dalloc(h, buffer_bytes) : nullptr;
     if (!d1) {  // without the memory the per-iteration kernels, which need none, do the solve
         if (d0) {
@@ -839,13 +754,10 @@ static int build_pcg(sim_handle *h)
         }
         return SIM_OK;
     }
-    host.resize(table_bytes);
-    dev = static_cast<unsigned char *>(d0);
-    tables();
+    std::vector<unsigned char> host(table_bytes);
+    pcg_place_tables(P, pd, host.data(), static_cast<unsigned char *>(d0), 0);
     CK(h, cudaMemcpy(d0, host.data(), table_bytes, cudaMemcpyHostToDevice));
-    dev = static_cast<unsigned char *>(d1);
-    buffers();
-    pd.has_diag = h->mat.dt > 0.0 || h->mat.k_contact > 0.0 ? 1 : 0;
+    pcg_place_buffers<T>(P, pd, static_cast<unsigned char *>(d1), 0);
     if (h->verbose)
         fprintf(stderr, "[softsim] persistent CG: %d CTAs%s x %d threads, %d slots, %d halo, %d coarse, %s, %d stages\n",
                 pd.n_cta, pd.cluster ? " (cluster)" : "", pd.threads, pd.ns, pd.max_halo, pd.n_coarse,
