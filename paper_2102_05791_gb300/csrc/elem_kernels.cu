@@ -27,6 +27,7 @@
 #include "reduce.cuh"
 #include "tma.cuh"
 #include "elem_math.cuh"
+#include "grid_sync.cuh"
 #include "pdl.cuh"
 #include "tile_device.cuh"
 
@@ -34,6 +35,44 @@ namespace softsim {
 
 // Per-vertex potential terms: gravity m g y and ground penalty kc max(0,-y)^p.
 __device__ __forceinline__ double pen_pow(double pen, int p) { return p == 2 ? pen * pen : pen * pen * pen; }
+
+// Gradient of one vertex's gravity, contact, inertia and friction added to
+// acc; with EN their energy to e[0] and its absolute value to e[1].
+template <int D, bool EN>
+__device__ __forceinline__ void add_vertex_terms(const VertDev &vd, const Phys &ph, int64_t gid, const double *u,
+                                                 const double *__restrict__ uhat, double acc[D], double *e)
+{
+    const double m = vd.mass[gid];
+    const double y = vd.X[gid * D + 1] + u[1];
+    const double pen = y < 0.0 ? -y : 0.0;
+    const double dcon = pen > 0.0 ? -ph.cpow * ph.kc * (ph.cpow == 2 ? pen : pen * pen) : 0.0;
+    acc[1] += ph.s_el * (m * ph.grav + dcon);
+    double w = 0.0, in = 0.0;
+    if (EN) w = ph.s_el * (m * ph.grav * y + (pen > 0.0 ? ph.kc * pen_pow(pen, ph.cpow) : 0.0));
+    if (EN) e[1] += fabs(w);
+    if (ph.dyn) {
+#pragma unroll
+        for (int c = 0; c < D; ++c) {
+            const double r = u[c] - uhat[gid * D + c];
+            acc[c] += m * r;
+            if (EN) in += 0.5 * m * r * r;
+        }
+        if (ph.fw) {
+            const double f = ph.fw[gid];
+#pragma unroll
+            for (int c = 0; c < D; ++c) {
+                if (c == 1) continue;
+                const double r = u[c] - ph.u0[gid * D + c];
+                acc[c] += f * r;
+                if (EN) in += 0.5 * f * r * r;
+            }
+        }
+    }
+    if (EN) {
+        e[0] += w + in;
+        e[1] += in;
+    }
+}
 
 // ---------------------------------------------------------------- energy
 
@@ -188,26 +227,71 @@ __global__ void __launch_bounds__(256) k_tile_energy(TileDev td, ElemDev<double>
 
 // ---------------------------------------------------------------- gradient
 
-template <int D>
+// Block sums of v[0..N) and minimum of mn, one tree for all; valid in thread 0.
+template <int N>
+__device__ __forceinline__ void block_sums_min(double (&v)[N], double &mn)
+{
+    __shared__ double red[N + 1][32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int q = 0; q < N; ++q) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+        mn = fmin(mn, __shfl_down_sync(0xffffffffu, mn, o));
+    }
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    __syncthreads();
+    if (lane == 0) {
+#pragma unroll
+        for (int q = 0; q < N; ++q) red[q][w] = v[q];
+        red[N][w] = mn;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < (int)(blockDim.x >> 5); ++k) {
+#pragma unroll
+            for (int q = 0; q < N; ++q) v[q] += red[q][k];
+            mn = fmin(mn, red[N][k]);
+        }
+    }
+}
+
+// Gradient of one tile and, with EN, its energy terms (energy, sum of their
+// absolute values, smallest J), FP64.
+//
+// What bounds it: the FP64 pipe (1/64 of the FP32 rate), about 230 operations a
+// tet.  Energy and gradient share the gathers, F, cof F, J and the logarithm,
+// so one pass gives both (393,216 tets: 352 us the call with a gradient and an
+// energy kernel of 167 + 143 us, 225 us with this one).  A mesh with fewer tiles than SMs splits each tile's elements
+// over a cluster of `split` CTAs: an element sends each corner's force to the
+// CTA that sums the corner's vertex (distributed shared memory), so the sums
+// keep their order.
+template <int D, bool EN>
 __global__ void __launch_bounds__(256) k_tile_grad(TileDev td, ElemDev<double> ed, VertDev vd, Phys ph,
                                                    const double *__restrict__ u, const double *__restrict__ uhat,
                                                    const double *__restrict__ a, double *__restrict__ g,
-                                                   double *__restrict__ hp, double *__restrict__ partials)
+                                                   double *__restrict__ hp, double *__restrict__ partials, int split)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     double *su = reinterpret_cast<double *>(smem);
     double *scr = su + td.max_tv * D;
-    const int t = blockIdx.x;
+    const int t = blockIdx.x / split, rank = blockIdx.x % split;
     const int es = td.tile_elem[t], ne_t = td.tile_elem[t + 1] - es;
     const int vs = td.tile_vert[t], nlv = td.tile_vert[t + 1] - vs;
+    // this CTA's share of the tile's elements and of its vertices
+    const int ech = (ne_t + split - 1) / split, vch = (nlv + split - 1) / split;
+    const int e0 = rank * ech, e1 = min(ne_t, e0 + ech), k0 = rank * vch, k1 = min(nlv, k0 + vch);
     for (int k = threadIdx.x; k < nlv; k += blockDim.x) {
         const int64_t gid = td.lv_gid[vs + k];
 #pragma unroll
         for (int c = 0; c < D; ++c) su[k * D + c] = u[gid * D + c];
     }
-    __syncthreads();
+    if (split > 1)
+        cluster_sync();  // every CTA of the cluster runs: its shared memory may be written
+    else
+        __syncthreads();
     const double mu = ph.mu, lam = ph.lam;
-    for (int le = threadIdx.x; le < ne_t; le += blockDim.x) {
+    double acc_e[3] = {0.0, 0.0, 0.0}, minJ = INFINITY;  // E, sum |terms|, |g|^2
+    for (int le = e0 + threadIdx.x; le < e1; le += blockDim.x) {
         const int64_t e = es + le;
         int lid[D + 1];
         unpack<D>(td.conn[e], lid);
@@ -219,7 +303,8 @@ __global__ void __launch_bounds__(256) k_tile_grad(TileDev td, ElemDev<double> e
         const double J = detF<double, D>(F, C);
         double l, cc, cp;
         log_terms<double>(ph.log_mode, mu, lam, J, l, cc, cp);
-        const double W = __ldg(ed.field(FI<D>::W) + e) * ph.s_el;
+        const double W0 = __ldg(ed.field(FI<D>::W) + e);
+        const double W = W0 * ph.s_el;
         double f[D], gv[D], Ff[D];
 #pragma unroll
         for (int i = 0; i < D; ++i) {
@@ -233,49 +318,72 @@ __global__ void __launch_bounds__(256) k_tile_grad(TileDev td, ElemDev<double> e
             for (int q = 0; q < D; ++q) s += F[i][q] * f[q];
             Ff[i] = s;
         }
-        double ka = ph.k * a[e];  // dpsi_m/dq = ka q
-        if (ph.muscle) {
-            double s2 = 0.0, c2;
+        const double av = a[e];
+        double ka = ph.k * av;  // dpsi_m/dq = ka q
+        double s2 = 0.0;
+        if (EN || ph.muscle) {
 #pragma unroll
             for (int i = 0; i < D; ++i) s2 += Ff[i] * Ff[i];
-            spring_terms<double>(W != 0.0, ph.k, a[e], sqrt(s2), ka, c2);
         }
+        if constexpr (EN) {
+            double I1 = 0.0;
+#pragma unroll
+            for (int i = 0; i < D; ++i)
+#pragma unroll
+                for (int j = 0; j < D; ++j) I1 += F[i][j] * F[i][j];
+            if (ph.log_mode == 0 && !(J > 0.0)) l = 0.0;
+            double musc = 0.5 * ka * s2;
+            if (ph.muscle) {
+                const double r = sqrt(s2) / av - 1.0;
+                musc = W0 != 0.0 ? 0.5 * ph.k * r * r : 0.0;
+            }
+            double w = W * (0.5 * mu * (I1 - D) - mu * l + 0.5 * lam * l * l + musc);
+            if (ph.log_mode == 0 && J <= 0.0) w = INFINITY;  // a NaN J (non-finite input) stays NaN
+            acc_e[0] += w;
+            acc_e[1] += fabs(w);
+            minJ = fmin(minJ, J);
+        }
+        if (ph.muscle) {
+            double c2;
+            spring_terms<double>(W != 0.0, ph.k, av, sqrt(s2), ka, c2);
+        }
+        const double muW = mu * W, ccW = cc * W, kaW = ka * W;
+#pragma unroll
+        for (int i = 0; i < D; ++i) Ff[i] *= kaW;
         double G[D][D];
 #pragma unroll
-        for (int i = 0; i < D; ++i)
+        for (int i = 0; i < D; ++i) {
+#pragma unroll
+            for (int k = 0; k < D; ++k) F[i][k] = muW * F[i][k] + ccW * C[i][k];
 #pragma unroll
             for (int j = 0; j < D; ++j) {
-                double s = 0.0;
+                double s = Ff[i] * gv[j];
 #pragma unroll
-                for (int k = 0; k < D; ++k) s += (mu * F[i][k] + cc * C[i][k]) * B[j][k];
-                G[i][j] = W * (s + ka * Ff[i] * gv[j]);
+                for (int k = 0; k < D; ++k) s += F[i][k] * B[j][k];
+                G[i][j] = s;
             }
-        store_corners<double, D>(scr + (int64_t)le * td.rs + corner_base(le), G);
+        }
+        double *rec = scr + (int64_t)le * td.rs + corner_base(le);
+        if (split == 1)
+            store_corners<double, D>(rec, G);
+        else
+            send_corners<D>(rec, G, lid, vch);
     }
-    __syncthreads();
+    if (split > 1)
+        cluster_sync();
+    else
+        __syncthreads();
+    pdl_trigger();  // the finalize kernel may be scheduled
     double gn2 = 0.0;
     const uint16_t *tinc = td.inc + (int64_t)es * (D + 1);
-    for (int k = threadIdx.x; k < nlv; k += blockDim.x) {
+    for (int k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
         const int code = td.lv_code[vs + k];
         if (code == LV_PAD) continue;
         double acc[D];
         gather_corners<double, D>(tinc, td.lv_inc[vs + k], scr, acc);
         const int64_t gid = td.lv_gid[vs + k];
         if (code == LV_INTERIOR) {
-            const double m = vd.mass[gid];
-            const double y = vd.X[gid * D + 1] + su[k * D + 1];
-            const double pen = y < 0.0 ? -y : 0.0;
-            const double dcon = pen > 0.0 ? -ph.cpow * ph.kc * (ph.cpow == 2 ? pen : pen * pen) : 0.0;
-            acc[1] += ph.s_el * (m * ph.grav + dcon);
-            if (ph.dyn)
-#pragma unroll
-                for (int c = 0; c < D; ++c) acc[c] += m * (su[k * D + c] - uhat[gid * D + c]);
-            if (ph.fw) {
-                const double f = ph.fw[gid];
-#pragma unroll
-                for (int c = 0; c < D; ++c)
-                    if (c != 1) acc[c] += f * (su[k * D + c] - ph.u0[gid * D + c]);
-            }
+            add_vertex_terms<D, EN>(vd, ph, gid, su + k * D, uhat, acc, acc_e);
             const bool fx = vd.fixed[gid] != 0;
 #pragma unroll
             for (int c = 0; c < D; ++c) {
@@ -288,41 +396,46 @@ __global__ void __launch_bounds__(256) k_tile_grad(TileDev td, ElemDev<double> e
             for (int c = 0; c < D; ++c) hp[(int64_t)(code >> 1) * D + c] = acc[c];
         }
     }
-    const double s = block_sum(gn2);
-    if (threadIdx.x == 0) partials[t] = s;
+    if constexpr (EN) {
+        acc_e[2] = gn2;
+        block_sums_min<3>(acc_e, minJ);
+        if (threadIdx.x == 0) {
+            double *p = partials + 4 * (size_t)blockIdx.x;
+            p[0] = acc_e[0];
+            p[1] = acc_e[1];
+            p[2] = acc_e[2];
+            p[3] = minJ;
+        }
+    } else {
+        const double s = block_sum(gn2);
+        if (threadIdx.x == 0) partials[blockIdx.x] = s;
+    }
 }
 
-template <int D>
+// Completes the gradient at halo vertices (their tiles' partial sums in tile
+// order plus the vertex terms); the last block sums the partials of both
+// kernels: [n_part] of the tile kernel, then one entry per block.
+template <int D, bool EN>
 __global__ void __launch_bounds__(256) k_fin_grad(TileDev td, VertDev vd, Phys ph, const double *__restrict__ u,
                                                   const double *__restrict__ uhat, const double *__restrict__ hp,
-                                                  double *__restrict__ g, double *__restrict__ partials,
+                                                  double *__restrict__ g, double *__restrict__ partials, int n_part,
                                                   DevScalars *__restrict__ sc)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    double gn2 = 0.0;
-    if (i < td.n_fin) {
-        const int64_t gid = td.fin_gid[i];
-        double acc[D];
+    const bool in = i < td.n_fin;
+    const int64_t gid = in ? td.fin_gid[i] : 0;
+    const int p0 = in ? td.fin_ptr[i] : 0, p1 = in ? td.fin_ptr[i + 1] : 0;
+    const bool fx = in && vd.fixed[gid] != 0;
+    pdl_wait();  // everything above is static
+    double gn2 = 0.0, acc_e[3] = {0.0, 0.0, 0.0}, minJ = INFINITY;
+    if (in) {
+        double acc[D], uv[D];
 #pragma unroll
-        for (int c = 0; c < D; ++c) acc[c] = 0.0;
-        for (int s = td.fin_ptr[i]; s < td.fin_ptr[i + 1]; ++s)
+        for (int c = 0; c < D; ++c) acc[c] = 0.0, uv[c] = u[gid * D + c];
+        for (int s = p0; s < p1; ++s)
 #pragma unroll
             for (int c = 0; c < D; ++c) acc[c] += hp[(int64_t)s * D + c];
-        const double m = vd.mass[gid];
-        const double y = vd.X[gid * D + 1] + u[gid * D + 1];
-        const double pen = y < 0.0 ? -y : 0.0;
-        const double dcon = pen > 0.0 ? -ph.cpow * ph.kc * (ph.cpow == 2 ? pen : pen * pen) : 0.0;
-        acc[1] += ph.s_el * (m * ph.grav + dcon);
-        if (ph.dyn)
-#pragma unroll
-            for (int c = 0; c < D; ++c) acc[c] += m * (u[gid * D + c] - uhat[gid * D + c]);
-        if (ph.fw) {
-            const double f = ph.fw[gid];
-#pragma unroll
-            for (int c = 0; c < D; ++c)
-                if (c != 1) acc[c] += f * (u[gid * D + c] - ph.u0[gid * D + c]);
-        }
-        const bool fx = vd.fixed[gid] != 0;
+        add_vertex_terms<D, EN>(vd, ph, gid, uv, uhat, acc, acc_e);
 #pragma unroll
         for (int c = 0; c < D; ++c) {
             const double o = fx ? 0.0 : acc[c];
@@ -330,12 +443,43 @@ __global__ void __launch_bounds__(256) k_fin_grad(TileDev td, VertDev vd, Phys p
             gn2 += o * o;
         }
     }
-    const double s = block_sum(gn2);
-    const int base = td.n_tiles;
-    if (threadIdx.x == 0) partials[base + blockIdx.x] = s;
-    if (last_block(&sc->ticket[TK_GRAD], gridDim.x)) {
-        const double tot = sum_partials(partials, base + gridDim.x);
-        if (threadIdx.x == 0) sc->gn2 = tot;
+    if constexpr (EN) {
+        acc_e[2] = gn2;
+        block_sums_min<3>(acc_e, minJ);
+        if (threadIdx.x == 0) {
+            double *p = partials + 4 * (size_t)(n_part + blockIdx.x);
+            p[0] = acc_e[0];
+            p[1] = acc_e[1];
+            p[2] = acc_e[2];
+            p[3] = minJ;
+        }
+        if (last_block(&sc->ticket[TK_GRAD], gridDim.x)) {
+            const double2 *p = reinterpret_cast<const double2 *>(partials);
+            double v[3] = {0.0, 0.0, 0.0}, mj = INFINITY;
+            const int n = n_part + gridDim.x;
+#pragma unroll 4
+            for (int k = threadIdx.x; k < n; k += blockDim.x) {
+                const double2 q0 = __ldcg(p + 2 * k), q1 = __ldcg(p + 2 * k + 1);
+                v[0] += q0.x;
+                v[1] += q0.y;
+                v[2] += q1.x;
+                mj = fmin(mj, q1.y);
+            }
+            block_sums_min<3>(v, mj);
+            if (threadIdx.x == 0) {
+                sc->E[0] = v[0];
+                sc->S[0] = v[1];
+                sc->gn2 = v[2];
+                sc->minJ = mj;
+            }
+        }
+    } else {
+        const double s = block_sum(gn2);
+        if (threadIdx.x == 0) partials[n_part + blockIdx.x] = s;
+        if (last_block(&sc->ticket[TK_GRAD], gridDim.x)) {
+            const double tot = sum_partials(partials, n_part + gridDim.x);
+            if (threadIdx.x == 0) sc->gn2 = tot;
+        }
     }
 }
 
@@ -676,19 +820,37 @@ void launch_energy(const Ctx &c, const Phys &ph, const double *u, const double *
         k_tile_energy<3><<<c.td.n_tiles, c.threads, sm, s>>>(c.td, c.e64, c.vd, ph, u, dir, uhat, a, tr, c.partials, c.sc);
 }
 
-void launch_grad(const Ctx &c, const Phys &ph, const double *u, const double *uhat, const double *a, double *g,
-                 double *hp, cudaStream_t s)
+// CTAs that share a tile: as many as leave every SM at most one (the FP64 pipe
+// is saturated by a tile's four warps, so more than one CTA an SM gains
+// nothing).  A backward-Euler step of 5,616 tets, 15 tiles: 3.51 -> 2.80 ms
+// together with the fused evaluation; 107 tiles stay whole.
+int eval_split(int n_tiles, int sms)
+{
+    int sp = 8;
+    while (sp > 1 && n_tiles * sp > sms) sp /= 2;
+    return sp;
+}
+
+template <int D, bool EN>
+static void grad_k(const Ctx &c, const Phys &ph, const double *u, const double *uhat, const double *a, double *g,
+                   double *hp, cudaStream_t s)
 {
     c.n_launch += 2;
     const size_t sm = smem_verts(c, sizeof(double), 1) + (size_t)c.td.max_te * c.td.rs * sizeof(double);
-    const int fb = c.n_fin_blocks;
-    if (c.dim == 2) {
-        k_tile_grad<2><<<c.td.n_tiles, c.threads, sm, s>>>(c.td, c.e64, c.vd, ph, u, uhat, a, g, hp, c.partials);
-        k_fin_grad<2><<<fb, 256, 0, s>>>(c.td, c.vd, ph, u, uhat, hp, g, c.partials, c.sc);
-    } else {
-        k_tile_grad<3><<<c.td.n_tiles, c.threads, sm, s>>>(c.td, c.e64, c.vd, ph, u, uhat, a, g, hp, c.partials);
-        k_fin_grad<3><<<fb, 256, 0, s>>>(c.td, c.vd, ph, u, uhat, hp, g, c.partials, c.sc);
-    }
+    const int n_part = c.td.n_tiles * c.split;
+    launch_cluster(c.split, k_tile_grad<D, EN>, dim3(n_part), dim3(c.threads), sm, s, c.td, c.e64, c.vd, ph, u, uhat,
+                   a, g, hp, c.partials, c.split);
+    launch_k(true, k_fin_grad<D, EN>, dim3(c.n_fin_blocks), dim3(256), 0, s, c.td, c.vd, ph, u, uhat,
+             (const double *)hp, g, c.partials, n_part, c.sc);
+}
+
+void launch_grad(const Ctx &c, const Phys &ph, const double *u, const double *uhat, const double *a, double *g,
+                 double *hp, bool energy, cudaStream_t s)
+{
+    if (c.dim == 2)
+        (energy ? grad_k<2, true> : grad_k<2, false>)(c, ph, u, uhat, a, g, hp, s);
+    else
+        (energy ? grad_k<3, true> : grad_k<3, false>)(c, ph, u, uhat, a, g, hp, s);
 }
 
 template <typename T>
@@ -826,8 +988,10 @@ cudaError_t configure_elem_kernels()
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, big)
     SET((k_tile_energy<2>));
     SET((k_tile_energy<3>));
-    SET((k_tile_grad<2>));
-    SET((k_tile_grad<3>));
+    SET((k_tile_grad<2, false>));
+    SET((k_tile_grad<3, false>));
+    SET((k_tile_grad<2, true>));
+    SET((k_tile_grad<3, true>));
 #define SET_HVP(T, MB)                                                       \
     SET((k_tile_hvp<T, 2, true, MB, 0, false>));                             \
     SET((k_tile_hvp<T, 3, true, MB, 0, false>));                             \

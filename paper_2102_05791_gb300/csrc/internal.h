@@ -165,6 +165,7 @@ struct Ctx {
     int muscle = 0;              // muscle model (the spring's HVP also stages the fiber)
     double *partials = nullptr;  // [n_partials] FP64 block partial sums
     int n_fin_blocks = 1;
+    int split = 1;               // CTAs (one cluster) per tile of the gradient kernel
     DevScalars *sc = nullptr;
     mutable int64_t n_launch = 0;  // kernels launched through this context
     mutable bool pdl = false;      // launch CG-loop kernels with programmatic dependent launch
@@ -181,9 +182,11 @@ void launch_energy(const Ctx &c, const Phys &ph, const double *u, const double *
                    cudaStream_t s);
 
 // FP64 gradient of the energy (with inertia when ph.dyn), masked; writes
-// sc->gn2 = |g|^2.  hp: halo scratch [n_slots][dim] double.
+// sc->gn2 = |g|^2, and with `energy` also sc->E[0], sc->S[0] and sc->minJ.
+// hp: halo scratch [n_slots][dim] double.
 void launch_grad(const Ctx &c, const Phys &ph, const double *u, const double *uhat,
-                 const double *a, double *g, double *hp, cudaStream_t s);
+                 const double *a, double *g, double *hp, bool energy, cudaStream_t s);
+int eval_split(int n_tiles, int sms);  // CTAs per tile of the gradient kernel
 
 // HVP y = A v (A = H, or M + dt^2 H when ph.dyn), masked; the activations
 // come from the element records.
@@ -227,6 +230,10 @@ template <typename T>
 void launch_hvp_cg(const Ctx &c, const Phys &ph, const T *u, const T *v, T *y, T *hp, cudaStream_t s);
 template <typename T>
 void launch_cg_dir(const Ctx &c, T *p, const T *r, cudaStream_t s);
+// First trial of a Newton step: up = u, u += d (and the FP32 copy), sc->gd =
+// g.d, sc->dir_fix = 1 when d is no descent direction.
+template <typename T>
+void launch_newton_step(const Ctx &c, const double *g, const T *d, double *u, double *up, float *u32, cudaStream_t s);
 template <typename T>
 void launch_dir_check(const Ctx &c, const double *g, T *d, cudaStream_t s);
 // *out = sum of the HVP tile kernel's v.Av partials, summed as k_cg_alpha does
@@ -240,9 +247,9 @@ void launch_x_to_u(const Ctx &c, const double *x, double *u, float *u32, const u
 void launch_u_to_x(const Ctx &c, const double *u, double *x, cudaStream_t s);
 void launch_uhat(const Ctx &c, const double *x0, const double *v0, double dt, double *uhat,
                  cudaStream_t s);
-template <typename T>
-// internal[e * stride] = user[perm[e]] (0 for padding elements), e in tile order
-void launch_gather_elem(const Ctx &c, const double *user, T *internal, cudaStream_t s, int64_t stride = 1);
+// The caller's activations in tile order (0 for padding elements): dense FP64,
+// and the activation slots of the FP64 and FP32 records; null: not wanted.
+void launch_set_activation(const Ctx &c, const double *user, double *a64, double *r64, float *r32, cudaStream_t s);
 template <typename Tin, typename Tout>
 void launch_convert(int64_t n, const Tin *in, Tout *out, cudaStream_t s);
 void launch_mask_copy(const Ctx &c, const double *in, double *out, cudaStream_t s);

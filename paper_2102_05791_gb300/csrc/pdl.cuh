@@ -39,4 +39,24 @@ inline cudaError_t launch_k(bool pdl, void (*k)(KArgs...), dim3 grid, dim3 block
     return cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);
 }
 
+// Launch with clusters of `size` consecutive CTAs.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_cluster(int size, void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                  Args &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = size;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = size > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);
+}
+
 }  // namespace softsim

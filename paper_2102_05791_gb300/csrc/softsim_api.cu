@@ -446,10 +446,13 @@ static int create_impl(sim_handle *h, const sim_mesh *mesh, const sim_material *
     c.muscle = h->mat.muscle_model;
     if (c.threads % 32 || c.threads > 256) return fail(h, SIM_EINVAL, "threads must be a multiple of 32, at most 256");
     c.n_fin_blocks = std::max(1, (td.n_fin + 255) / 256);
+    int n_sm = 0;
+    CK(h, cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, h->device));
+    c.split = eval_split(td.n_tiles, n_sm);
 
     // --- work buffers
     const int64_t nd = nv * d;
-    const int n_part = std::max({td.n_tiles + c.n_fin_blocks, vec_grid_size(nd), vec_grid_size(ne_int),
+    const int n_part = std::max({td.n_tiles * c.split + c.n_fin_blocks, vec_grid_size(nd), vec_grid_size(ne_int),
                                   cg_update_grid_size(nv), 1});
     c.partials = (double *)dalloc(h, sizeof(double) * (size_t)n_part * (2 * kMaxTrials + 1));
     h->sc = (DevScalars *)dalloc(h, sizeof(DevScalars));
@@ -557,14 +560,18 @@ struct View<double> {
     static double *hp(sim_handle *h) { return h->hp64; }
 };
 
-// Set the internal activation copies from the caller's array.
-static int set_activation(sim_handle *h, const double *a, cudaStream_t s)
+// The copies of the caller's activations a call reads.  A record's slot is 4
+// or 8 bytes of a record of its own sectors (31 us each at 3.1 million tets),
+// so only what is read is written.
+enum { ACT_DENSE = 1, ACT_REC = 2, ACT_REC64 = 4 };  // FP64 array; records of the handle's precision; FP64 records
+
+static int set_activation(sim_handle *h, const double *a, int what, cudaStream_t s)
 {
     const Ctx &c = h->ctx;
     const int slot = hvp_fields(c.dim, c.muscle == SIM_MUSCLE_SPRING);  // after the HVP fields
-    launch_gather_elem<double>(c, a, h->a64, s);
-    launch_gather_elem<double>(c, a, c.rec64 + slot, s, c.td.rs);
-    if (is_mixed(h)) launch_gather_elem<float>(c, a, c.rec32 + slot, s, c.td.rs);
+    const bool r64 = (what & ACT_REC64) || (!is_mixed(h) && (what & ACT_REC)), r32 = is_mixed(h) && (what & ACT_REC);
+    launch_set_activation(c, a, what & ACT_DENSE ? h->a64 : nullptr, r64 ? c.rec64 + slot : nullptr,
+                          r32 ? c.rec32 + slot : nullptr, s);
     CKL(h);
     return SIM_OK;
 }
@@ -845,8 +852,8 @@ static int newton_impl(sim_handle *h, bool dyn, sim_solve_stats *st, cudaStream_
     int rc;
     const double *uh = dyn ? h->uhat : nullptr;
     const double t0 = 0.0;
-    launch_grad(c, ph, h->u, uh, h->a64, h->g, h->hp64, s);
-    launch_energy(c, ph, h->u, nullptr, uh, h->a64, &t0, 1, s);
+    double *u_prev = h->Hx;  // the state before the step (FP64 vector of the adjoint, unused here)
+    launch_grad(c, ph, h->u, uh, h->a64, h->g, h->hp64, true, s);
     CKL(h);
     if ((rc = read_scalars(h, s))) return rc;
     double gn = std::sqrt(h->sc_host->gn2);
@@ -880,58 +887,75 @@ static int newton_impl(sim_handle *h, bool dyn, sim_solve_stats *st, cudaStream_
             CKL(h);
             if ((rc = run_cg<T>(h, ph, h->opt.max_cg, s))) return rc;
         }
-        launch_dir_check<T>(c, h->g, (T *)h->vd, s);
+        // line search: t = 1, taken and evaluated in full (energy and gradient
+        // share their work); on rejection undone, then batches of halvings
+        launch_newton_step<T>(c, h->g, (const T *)h->vd, h->u, u_prev, h->u32, s);
+        launch_grad(c, ph, h->u, uh, h->a64, h->g, h->hp64, true, s);
         CKL(h);
-        // line search: t = 1, then batches of halvings
-        bool ok = false;
+        if ((rc = read_scalars(h, s))) return rc;
+        S.cg_iters_total += h->sc_host->iter;
+        bool ok = false, fix = h->sc_host->dir_fix != 0;
         double t_acc = 0.0, E_acc = 0.0, S_acc = 0.0;
+        auto accept = [&](int j, double t, int slot) {
+            const double Et = h->sc_host->E[slot], St = h->sc_host->S[slot];
+            const double slack = 64.0 * eps * std::max(Sabs, St);
+            if (!std::isfinite(Et) || !(Et <= E + 1e-4 * t * h->sc_host->gd + slack)) return false;
+            t_acc = t;
+            E_acc = Et;
+            S_acc = St;
+            S.ls_halvings += j;
+            return true;
+        };
         int j0 = 0;
-        const double *dir64 = nullptr;
-        if (is_mixed(h)) {
-            launch_convert<float, double>(c.nv * c.dim, (const float *)h->vd, h->work, s);
-            c.n_launch += 1;
-            dir64 = h->work;
-        } else {
-            dir64 = (const double *)h->vd;
+        if (!fix && h->opt.max_ls > 0) {
+            ok = accept(0, 1.0, 0);
+            j0 = 1;
         }
-        while (j0 < h->opt.max_ls && !ok) {
-            const int nt = j0 == 0 ? 1 : std::min(kMaxTrials, h->opt.max_ls - j0);
-            double ts[kMaxTrials];
-            for (int j = 0; j < nt; ++j) ts[j] = std::ldexp(1.0, -(j0 + j));
-            launch_energy(c, ph, h->u, dir64, uh, h->a64, ts, nt, s);
-            CKL(h);
-            if ((rc = read_scalars(h, s))) return rc;
-            const double gd = h->sc_host->gd;
-            if (j0 == 0) S.cg_iters_total += h->sc_host->iter;
-            for (int j = 0; j < nt; ++j) {
-                const double Et = h->sc_host->E[j], St = h->sc_host->S[j];
-                const double slack = 64.0 * eps * std::max(Sabs, St);
-                if (std::isfinite(Et) && Et <= E + 1e-4 * ts[j] * gd + slack) {
-                    ok = true;
-                    t_acc = ts[j];
-                    E_acc = Et;
-                    S_acc = St;
-                    S.ls_halvings += j0 + j;
-                    break;
-                }
+        if (!ok) {
+            CK(h, cudaMemcpyAsync(h->u, u_prev, sizeof(double) * c.nv * c.dim, cudaMemcpyDeviceToDevice, s));
+            if (fix) {  // no descent direction: d := -g
+                launch_grad(c, ph, h->u, uh, h->a64, h->g, h->hp64, false, s);
+                launch_dir_check<T>(c, h->g, (T *)h->vd, s);
             }
-            if (!ok) j0 += nt;
+            const double *dir64 = (const double *)h->vd;
+            if (is_mixed(h)) {
+                launch_convert<float, double>(c.nv * c.dim, (const float *)h->vd, h->work, s);
+                launch_convert<double, float>(c.nv * c.dim, h->u, h->u32, s);
+                c.n_launch += 2;
+                dir64 = h->work;
+            }
+            while (j0 < h->opt.max_ls && !ok) {
+                const int nt = j0 == 0 ? 1 : std::min(kMaxTrials, h->opt.max_ls - j0);
+                double ts[kMaxTrials];
+                for (int j = 0; j < nt; ++j) ts[j] = std::ldexp(1.0, -(j0 + j));
+                launch_energy(c, ph, h->u, dir64, uh, h->a64, ts, nt, s);
+                CKL(h);
+                if ((rc = read_scalars(h, s))) return rc;
+                for (int j = 0; j < nt && !ok; ++j) ok = accept(j0 + j, ts[j], j);
+                if (!ok) j0 += nt;
+            }
+            if (ok) {
+                launch_step_update<T>(c, h->u, (const T *)h->vd, t_acc, h->u32, s);
+                launch_grad(c, ph, h->u, uh, h->a64, h->g, h->hp64, true, s);
+                CKL(h);
+                if ((rc = read_scalars(h, s))) return rc;
+            }
         }
         if (!ok) {
             if (h->verbose) fprintf(stderr, "[softsim] newton %d: line search failed, |g|/|g0| %.3e\n", it, gn / g0);
             S.ls_halvings += h->opt.max_ls;
             S.status = SIM_ELINESEARCH;
+            // the smallest J of the state that stays
+            launch_energy(c, ph, h->u, nullptr, uh, h->a64, &t0, 1, s);
+            CKL(h);
+            if ((rc = read_scalars(h, s))) return rc;
             break;
         }
         if (h->verbose)
             fprintf(stderr, "[softsim] newton %d: |g|/|g0| %.3e, eta %.2e, cg %d%s, t %.3g, E %.10e\n", it, gn / g0, eta,
-                    h->sc_host->iter, h->sc_host->dir_fix ? " (steepest descent)" : "", t_acc, E_acc);
-        launch_step_update<T>(c, h->u, (const T *)h->vd, t_acc, h->u32, s);
+                    h->sc_host->iter, fix ? " (steepest descent)" : "", t_acc, E_acc);
         E = E_acc;
         Sabs = S_acc;
-        launch_grad(c, ph, h->u, uh, h->a64, h->g, h->hp64, s);
-        CKL(h);
-        if ((rc = read_scalars(h, s))) return rc;
         gn = std::sqrt(h->sc_host->gn2);
         if (!std::isfinite(gn)) {
             S.status = SIM_ENAN;
@@ -940,10 +964,7 @@ static int newton_impl(sim_handle *h, bool dyn, sim_solve_stats *st, cudaStream_
     }
     S.newton_iters = it;
     S.res_final = gn;
-    launch_energy(c, ph, h->u, nullptr, uh, h->a64, &t0, 1, s);
-    CKL(h);
-    if ((rc = read_scalars(h, s))) return rc;
-    S.min_J = h->sc_host->minJ;
+    S.min_J = h->sc_host->minJ;  // of the last state evaluated in full
     if (st) *st = S;
     return S.status;
 }
@@ -1048,12 +1069,12 @@ extern "C" int sim_energy_grad(sim_handle *h, const double *x, const double *a, 
     cudaStream_t s = (cudaStream_t)stream;
     int rc;
     if ((rc = set_state(h, x, false, s))) return rc;
-    if ((rc = set_activation(h, a, s))) return rc;
+    if ((rc = set_activation(h, a, ACT_DENSE, s))) return rc;
     const Phys ph = make_phys(h, false);
-    if (grad) launch_grad(h->ctx, ph, h->u, nullptr, h->a64, grad, h->hp64, s);
+    if (grad) launch_grad(h->ctx, ph, h->u, nullptr, h->a64, grad, h->hp64, E_dev != nullptr, s);
     if (E_dev) {
         const double t0 = 0.0;
-        launch_energy(h->ctx, ph, h->u, nullptr, nullptr, h->a64, &t0, 1, s);
+        if (!grad) launch_energy(h->ctx, ph, h->u, nullptr, nullptr, h->a64, &t0, 1, s);
         CK(h, cudaMemcpyAsync(E_dev, &h->sc->E[0], sizeof(double), cudaMemcpyDeviceToDevice, s));
     }
     CKL(h);
@@ -1067,7 +1088,7 @@ extern "C" int sim_hvp(sim_handle *h, const double *x, const double *a, const vo
     cudaStream_t s = (cudaStream_t)stream;
     int rc;
     if ((rc = set_state(h, x, false, s))) return rc;
-    if ((rc = set_activation(h, a, s))) return rc;
+    if ((rc = set_activation(h, a, ACT_REC, s))) return rc;
     const Phys ph = make_phys(h, false);
     if (is_mixed(h))
         launch_hvp<float>(h->ctx, ph, h->u32, (const float *)v, (float *)Hv, h->hp32, s);
@@ -1106,7 +1127,7 @@ extern "C" int sim_hvp_dot(sim_handle *h, const double *x, const double *a, cons
     cudaStream_t s = (cudaStream_t)stream;
     int rc;
     if ((rc = set_state(h, x, false, s))) return rc;
-    if ((rc = set_activation(h, a, s))) return rc;
+    if ((rc = set_activation(h, a, ACT_REC, s))) return rc;
     return is_mixed(h) ? hvp_dot_impl<float>(h, v, Hv, vHv, s) : hvp_dot_impl<double>(h, v, Hv, vHv, s);
 }
 
@@ -1122,7 +1143,7 @@ extern "C" int sim_newton_solve(sim_handle *h, const double *x_init, const doubl
     if (!x_init) return fail(h, SIM_EINVAL, "null x_init");
     cudaStream_t s = (cudaStream_t)stream;
     int rc;
-    if ((rc = set_activation(h, a, s))) return rc;
+    if ((rc = set_activation(h, a, ACT_DENSE | ACT_REC, s))) return rc;
     if (dyn) launch_uhat(h->ctx, x0, v0, h->mat.dt, h->uhat, s);
     if (dyn && h->fw) launch_friction_prep(h->ctx, x0, h->mat.k_friction, h->mat.eps_friction, h->u0, h->fw, s);
     if ((rc = set_state(h, x_init, true, s))) return rc;
@@ -1143,7 +1164,7 @@ extern "C" int sim_adjoint_solve(sim_handle *h, const double *x_star, const doub
     cudaStream_t s = (cudaStream_t)stream;
     int rc;
     if ((rc = set_state(h, x_star, false, s))) return rc;
-    if ((rc = set_activation(h, a, s))) return rc;
+    if ((rc = set_activation(h, a, ACT_REC | ACT_REC64, s))) return rc;
     const bool dyn = h->mat.dt > 0.0;
     const int status = is_mixed(h) ? adjoint_impl<float>(h, dyn, dLdx, lambda, st, s)
                                    : adjoint_impl<double>(h, dyn, dLdx, lambda, st, s);
@@ -1161,7 +1182,7 @@ extern "C" int sim_param_vjp(sim_handle *h, const double *x_star, const double *
     cudaStream_t s = (cudaStream_t)stream;
     int rc;
     if ((rc = set_state(h, x_star, false, s))) return rc;
-    if ((rc = set_activation(h, a, s))) return rc;
+    if ((rc = set_activation(h, a, ACT_DENSE, s))) return rc;
     const Phys ph = make_phys(h, h->mat.dt > 0.0);
     launch_param_vjp(h->ctx, ph, h->u, h->a64, lambda, dLda, s);
     CKL(h);
@@ -1177,7 +1198,7 @@ extern "C" int sim_material_vjp(sim_handle *h, const double *x_star, const doubl
     cudaStream_t s = (cudaStream_t)stream;
     int rc;
     if ((rc = set_state(h, x_star, false, s))) return rc;
-    if ((rc = set_activation(h, a, s))) return rc;
+    if ((rc = set_activation(h, a, ACT_DENSE, s))) return rc;
     const Phys ph = make_phys(h, h->mat.dt > 0.0);
     launch_material_vjp(h->ctx, ph, h->u, h->a64, lambda, dLdmu, dLdlambda, dLdk, s);
     CKL(h);

@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include "elem_math.cuh"
+#include "grid_sync.cuh"
 #include "internal.h"
 
 namespace softsim {
@@ -34,6 +35,31 @@ __device__ __forceinline__ void store_corners(T *rec, const T G[D][D])
             reinterpret_cast<float2 *>(rec)[q] = make_float2(out[2 * q], out[2 * q + 1]);
         else
             reinterpret_cast<double2 *>(rec)[q] = make_double2(out[2 * q], out[2 * q + 1]);
+    }
+}
+
+// The same corner forces, FP64, each sent to the same slot of the CTA of the
+// cluster that sums the corner's vertex (vch local vertices per CTA).
+template <int D>
+__device__ __forceinline__ void send_corners(const double *rec, const double G[D][D], const int lid[D + 1], int vch)
+{
+#pragma unroll
+    for (int k = 0; k <= D; ++k) {
+        double v[D];
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+            if (k > 0) {
+                v[i] = G[i][k - 1];
+            } else {
+                v[i] = 0.0;
+#pragma unroll
+                for (int j = 0; j < D; ++j) v[i] -= G[i][j];
+            }
+        }
+        const uint32_t at = dsmem_addr(rec + k * D, (uint32_t)(lid[k] / vch));
+#pragma unroll
+        for (int i = 0; i < D; ++i)
+            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(at + 8u * i), "d"(v[i]) : "memory");
     }
 }
 
