@@ -19,7 +19,7 @@ namespace softsim {
 // One thread per element: its corner pairs' blocks to their contribution
 // slots.  Bound by the scattered 36-byte (FP32) writes.
 template <typename T, int D, bool SPRING>
-__global__ void __launch_bounds__(256) k_asm_elem(TileDev td, const T *__restrict__ erec, Phys ph,
+__global__ void __launch_bounds__(256) k_asm_elem(TileDev td, const T *__restrict__ erec, const T *__restrict__ act, Phys ph,
                                                   const T *__restrict__ u, const uint32_t *__restrict__ cpos,
                                                   T *__restrict__ contrib)
 {
@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(256) k_asm_elem(TileDev td, const T *__restric
             for (int j = 0; j < D; ++j) B[i][j] = rv[FI<D>::B + i * D + j];
         }
         edges<T, D>(su, lid, Du);
-        elem_blocks<T, D>(B, gv, f, rv[FI<D>::W] * sel, rv[NF], Du, SPRING, ph.log_mode, mu, lam, kk, cpos + e * NP,
+        elem_blocks<T, D>(B, gv, f, rv[FI<D>::W] * sel, act[e], Du, SPRING, ph.log_mode, mu, lam, kk, cpos + e * NP,
                           contrib);
     }
 }
@@ -222,12 +222,13 @@ static void assemble(const Ctx &c, const PcgDev &pd, const Phys &ph, const T *u,
                      cudaStream_t s)
 {
     const T *er = sizeof(T) == 4 ? reinterpret_cast<const T *>(c.rec32) : reinterpret_cast<const T *>(c.rec64);
+    const T *ac = sizeof(T) == 4 ? reinterpret_cast<const T *>(c.a32) : reinterpret_cast<const T *>(c.a64);
     const size_t sm = (size_t)c.td.max_tv * D * sizeof(T);
     T *contrib = static_cast<T *>(pd.contrib), *blk = static_cast<T *>(pd.blk);
     if (c.muscle)
-        k_asm_elem<T, D, true><<<c.td.n_tiles, c.threads, sm, s>>>(c.td, er, ph, u, pd.cpos, contrib);
+        k_asm_elem<T, D, true><<<c.td.n_tiles, c.threads, sm, s>>>(c.td, er, ac, ph, u, pd.cpos, contrib);
     else
-        k_asm_elem<T, D, false><<<c.td.n_tiles, c.threads, sm, s>>>(c.td, er, ph, u, pd.cpos, contrib);
+        k_asm_elem<T, D, false><<<c.td.n_tiles, c.threads, sm, s>>>(c.td, er, ac, ph, u, pd.cpos, contrib);
     k_asm_edge<T, D><<<(unsigned)((pd.n_edges + 255) / 256), 256, 0, s>>>(pd.n_edges, pd.edge_ptr, contrib, blk);
     const dim3 gs((unsigned)pd.n_chunks, pd.tpr ? (unsigned)((pd.max_entries + 255) / 256) : 1u);
     k_asm_slice<T, D><<<gs, 256, 0, s>>>(pd.n_edges, pd.chunk_ent, pd.ent_idx, pd.ent_edge, blk,

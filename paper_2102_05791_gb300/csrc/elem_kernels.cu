@@ -514,12 +514,21 @@ struct HvpSmem {
 // per local vertex adds its corners in fixed order.
 // SPRING selects the active-spring muscle at compile time, so the
 // contractile kernel carries none of its code or its extra fields.
-template <typename T, int D, bool CG, int MINB, int MTE, bool SPRING>
+// MODE: HVP_STATE reads the displacement u and the activations in tile order,
+// HVP_CG also forms p.Ap, and HVP_CALLER takes positions x and activations as
+// the caller has them (u = x - X rounded to T while staging), which saves a
+// small mesh one launch.  A thread fetches its elements' activations before the
+// wait for the records and puts them into its records.
+enum HvpMode { HVP_STATE, HVP_CG, HVP_CALLER };
+
+template <typename T, int D, int MODE, int MINB, int MTE, bool SPRING>
 __global__ void __launch_bounds__(256, MINB) k_tile_hvp(TileDev td, const T *__restrict__ erec, VertDev vd,
-                                                  Phys ph, const T *__restrict__ u, const T *__restrict__ v,
+                                                  Phys ph, const T *__restrict__ u, const double *__restrict__ x,
+                                                  const void *__restrict__ act, const T *__restrict__ v,
                                                   T *__restrict__ y, T *__restrict__ hp,
                                                   double *__restrict__ partials, DevScalars *__restrict__ sc)
 {
+    constexpr bool CG = MODE == HVP_CG;
     extern __shared__ __align__(128) unsigned char smem[];
     // MTE != 0: the tile capacity is a compile-time constant, so every
     // record and corner offset below folds into an immediate
@@ -559,6 +568,21 @@ __global__ void __launch_bounds__(256, MINB) k_tile_hvp(TileDev td, const T *__r
     // Everything copied so far is static during a solve; state (u, v) and the
     // CG scalars are read only after the predecessor kernel has completed.
     pdl_wait();
+    constexpr int PRE = 4;  // activations a thread holds (tiles of more than PRE x threads elements: the rest later)
+    T av[PRE];
+    auto activation = [&](int le) {
+        if constexpr (MODE == HVP_CALLER) {
+            const int32_t pe = td.perm[es + le];
+            return pe >= 0 ? T(static_cast<const double *>(act)[pe]) : T(0);
+        } else {
+            return static_cast<const T *>(act)[es + le];
+        }
+    };
+#pragma unroll
+    for (int j = 0; j < PRE; ++j) {
+        const int le = threadIdx.x + j * blockDim.x;
+        av[j] = le < ne_t ? activation(le) : T(0);
+    }
     // the flag is read before the wait so that its load overlaps the copies
     // in flight; the previous kernel has completed, so every thread reads the
     // same value
@@ -585,6 +609,9 @@ __global__ void __launch_bounds__(256, MINB) k_tile_hvp(TileDev td, const T *__r
             suv[k * 6 + 0] = u4.x;
             suv[k * 6 + 1] = u4.y;
             suv[k * 6 + 2] = u4.z;
+        } else if constexpr (MODE == HVP_CALLER) {
+#pragma unroll
+            for (int c = 0; c < D; ++c) suv[k * 2 * D + c] = T(x[gid * D + c] - vd.X[gid * D + c]);
         } else {
 #pragma unroll
             for (int c = 0; c < D; ++c) suv[k * 2 * D + c] = u[gid * D + c];
@@ -599,6 +626,13 @@ __global__ void __launch_bounds__(256, MINB) k_tile_hvp(TileDev td, const T *__r
         }
         return;
     }
+    // each thread's own elements: no barrier needed
+#pragma unroll
+    for (int j = 0; j < PRE; ++j) {
+        const int le = threadIdx.x + j * blockDim.x;
+        if (le < ne_t) sRec[le * RS + NF] = av[j];
+    }
+    for (int le = threadIdx.x + PRE * blockDim.x; le < ne_t; le += blockDim.x) sRec[le * RS + NF] = activation(le);
     const T mu = pick<T>(ph.mu, ph.mu_f), lam = pick<T>(ph.lam, ph.lam_f);
     const T sel = pick<T>(ph.s_el, ph.s_el_f), kk = pick<T>(ph.k, ph.k_f);
     // CG: p.Ap of this tile from the element quadratic forms v_e . (H_e v_e)
@@ -622,26 +656,41 @@ __global__ void __launch_bounds__(256, MINB) k_tile_hvp(TileDev td, const T *__r
 }
 
 // Completes y = A v at halo vertices: the tiles' partial sums in tile order
-// plus the per-vertex terms.
+// plus the per-vertex terms.  x: the caller's positions (HVP_CALLER; u unused).
+// Latency of a few dependent loads: the table entries come before the wait for
+// the tile kernel, and the partial sums four at a time.
 template <typename T, int D>
 __global__ void __launch_bounds__(256) k_fin_hvp(TileDev td, VertDev vd, Phys ph, const T *__restrict__ u,
-                                                 const T *__restrict__ v, const T *__restrict__ hp, T *__restrict__ y)
+                                                 const double *__restrict__ x, const T *__restrict__ v,
+                                                 const T *__restrict__ hp, T *__restrict__ y)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= td.n_fin) return;
-    const int64_t gid = td.fin_gid[i];
-    const bool fx = vd.fixed[gid] != 0;
-    T acc[D];
-#pragma unroll
-    for (int c = 0; c < D; ++c) acc[c] = T(0);
-    for (int s = td.fin_ptr[i]; s < td.fin_ptr[i + 1]; ++s)
-#pragma unroll
-        for (int c = 0; c < D; ++c) acc[c] += hp[(int64_t)s * D + c];
+    const bool in = i < td.n_fin;
+    const int64_t gid = in ? td.fin_gid[i] : 0;
+    const int s0 = in ? td.fin_ptr[i] : 0, s1 = in ? td.fin_ptr[i + 1] : 0;
+    const bool fx = in && vd.fixed[gid] != 0;
+    pdl_wait();  // everything above is static
+    if (!in) return;
     T vv[D];
 #pragma unroll
     for (int c = 0; c < D; ++c) vv[c] = fx ? T(0) : v[gid * D + c];
+    T acc[D];
+#pragma unroll
+    for (int c = 0; c < D; ++c) acc[c] = T(0);
+    for (int s = s0; s < s1; s += 4) {
+        T h[4][D];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int c = 0; c < D; ++c) h[q][c] = s + q < s1 ? hp[(int64_t)(s + q) * D + c] : T(0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int c = 0; c < D; ++c) acc[c] += h[q][c];
+    }
     if (ph.kc > 0.0) {
-        const double yy = vd.X[gid * D + 1] + (double)u[gid * D + 1];
+        const double ux = x ? (double)T(x[gid * D + 1] - vd.X[gid * D + 1]) : (double)u[gid * D + 1];
+        const double yy = vd.X[gid * D + 1] + ux;
         const double pen = yy < 0.0 ? -yy : 0.0;
         const double d2 = pen > 0.0 ? ph.cpow * (ph.cpow - 1) * ph.kc * (ph.cpow == 2 ? 1.0 : pen) : 0.0;
         acc[1] += T(ph.s_el * d2) * vv[1];
@@ -861,6 +910,13 @@ template <>
 const double *erec<double>(const Ctx &c) { return c.rec64; }
 
 template <typename T>
+static const T *eact(const Ctx &c);
+template <>
+const float *eact<float>(const Ctx &c) { return c.a32; }
+template <>
+const double *eact<double>(const Ctx &c) { return c.a64; }
+
+template <typename T>
 size_t hvp_smem(const Ctx &c)
 {
     return c.dim == 2 ? HvpSmem<T, 2>(c.td.max_te, c.td.max_tv, c.td.rs).total
@@ -884,76 +940,97 @@ int hvp_blocks_per_sm(const Ctx &c)
 // Tile capacities with a compile-time specialisation (the library defaults).
 constexpr int kCap2 = 512, kCap3 = 384;
 
-template <typename T, int D, bool CG, int MINB>
-static void hvp_tile_v(const Ctx &c, const Phys &ph, const T *u, const T *v, T *y, T *hp, cudaStream_t s)
+// What an HVP reads besides v: the handle's displacement and activations, or
+// (x set) the caller's positions and activations.
+template <typename T>
+struct HvpIn {
+    const T *u;
+    const double *x;
+    const void *act;
+};
+
+template <typename T, int D, int MODE, int MINB>
+static void hvp_tile_v(const Ctx &c, const Phys &ph, const HvpIn<T> &in, const T *v, T *y, T *hp, cudaStream_t s)
 {
     constexpr int CAP = D == 2 ? kCap2 : kCap3;
+    auto go = [&](auto k) {
+        launch_k(c.pdl, k, dim3(c.td.n_tiles), dim3(c.threads), hvp_smem<T>(c), s, c.td, erec<T>(c), c.vd, ph, in.u,
+                 in.x, in.act, v, y, hp, c.partials, c.sc);
+    };
     if (c.muscle)  // the spring variant exists for the runtime tile capacity only
-        launch_k(c.pdl, k_tile_hvp<T, D, CG, MINB, 0, true>, dim3(c.td.n_tiles), dim3(c.threads), hvp_smem<T>(c), s,
-                 c.td, erec<T>(c), c.vd, ph, u, v, y, hp, c.partials, c.sc);
+        go(k_tile_hvp<T, D, MODE, MINB, 0, true>);
     else if (sizeof(T) == 4 && c.td.max_te == CAP)
-        launch_k(c.pdl, k_tile_hvp<T, D, CG, MINB, (sizeof(T) == 4 ? CAP : 0), false>, dim3(c.td.n_tiles),
-                 dim3(c.threads), hvp_smem<T>(c), s, c.td, erec<T>(c), c.vd, ph, u, v, y, hp, c.partials, c.sc);
+        go(k_tile_hvp<T, D, MODE, MINB, (sizeof(T) == 4 ? CAP : 0), false>);
     else
-        launch_k(c.pdl, k_tile_hvp<T, D, CG, MINB, 0, false>, dim3(c.td.n_tiles), dim3(c.threads), hvp_smem<T>(c), s,
-                 c.td, erec<T>(c), c.vd, ph, u, v, y, hp, c.partials, c.sc);
+        go(k_tile_hvp<T, D, MODE, MINB, 0, false>);
 }
 
-template <typename T, bool CG>
-static void hvp_tile(const Ctx &c, const Phys &ph, const T *u, const T *v, T *y, T *hp, cudaStream_t s)
+template <typename T, int MODE>
+static void hvp_tile(const Ctx &c, const Phys &ph, const HvpIn<T> &in, const T *v, T *y, T *hp, cudaStream_t s)
 {
     c.n_launch += 1;
     const int b = hvp_blocks_per_sm<T>(c);
     if constexpr (sizeof(T) == 4) {
         if (c.dim == 2)
-            (b >= 4 ? hvp_tile_v<T, 2, CG, 4> : hvp_tile_v<T, 2, CG, 3>)(c, ph, u, v, y, hp, s);
+            (b >= 4 ? hvp_tile_v<T, 2, MODE, 4> : hvp_tile_v<T, 2, MODE, 3>)(c, ph, in, v, y, hp, s);
         else
             // the CG variant also forms p.Ap: at 64 registers it spilled, at
             // the 3-CTA bound it takes 72, which still lets 7 of the
             // 128-thread tiles be resident (shared memory allows 7)
-            ((b >= 4 && !CG) ? hvp_tile_v<T, 3, CG, 4> : hvp_tile_v<T, 3, CG, 3>)(c, ph, u, v, y, hp, s);
+            ((b >= 4 && MODE == HVP_STATE) ? hvp_tile_v<T, 3, MODE, 4> : hvp_tile_v<T, 3, MODE, 3>)(c, ph, in, v, y, hp,
+                                                                                                 s);
     } else {
         if (c.dim == 2)
-            (b >= 2 ? hvp_tile_v<T, 2, CG, 2> : hvp_tile_v<T, 2, CG, 1>)(c, ph, u, v, y, hp, s);
+            (b >= 2 ? hvp_tile_v<T, 2, MODE, 2> : hvp_tile_v<T, 2, MODE, 1>)(c, ph, in, v, y, hp, s);
         else
-            (b >= 2 ? hvp_tile_v<T, 3, CG, 2> : hvp_tile_v<T, 3, CG, 1>)(c, ph, u, v, y, hp, s);
+            (b >= 2 ? hvp_tile_v<T, 3, MODE, 2> : hvp_tile_v<T, 3, MODE, 1>)(c, ph, in, v, y, hp, s);
     }
 }
 
 template <typename T>
-static void hvp_fin(const Ctx &c, const Phys &ph, const T *u, const T *v, T *y, const T *hp, cudaStream_t s)
+static void hvp_fin(const Ctx &c, const Phys &ph, const HvpIn<T> &in, const T *v, T *y, const T *hp, cudaStream_t s)
 {
     c.n_launch += 1;
     if (c.dim == 2)
-        k_fin_hvp<T, 2><<<c.n_fin_blocks, 256, 0, s>>>(c.td, c.vd, ph, u, v, hp, y);
+        launch_k(true, k_fin_hvp<T, 2>, dim3(c.n_fin_blocks), dim3(256), 0, s, c.td, c.vd, ph, in.u, in.x, v, hp, y);
     else
-        k_fin_hvp<T, 3><<<c.n_fin_blocks, 256, 0, s>>>(c.td, c.vd, ph, u, v, hp, y);
+        launch_k(true, k_fin_hvp<T, 3>, dim3(c.n_fin_blocks), dim3(256), 0, s, c.td, c.vd, ph, in.u, in.x, v, hp, y);
 }
 
 template <typename T>
 void launch_hvp(const Ctx &c, const Phys &ph, const T *u, const T *v, T *y, T *hp, cudaStream_t s)
 {
-    hvp_tile<T, false>(c, ph, u, v, y, hp, s);
-    hvp_fin<T>(c, ph, u, v, y, hp, s);
+    const HvpIn<T> in{u, nullptr, eact<T>(c)};
+    hvp_tile<T, HVP_STATE>(c, ph, in, v, y, hp, s);
+    hvp_fin<T>(c, ph, in, v, y, hp, s);
+}
+
+template <typename T>
+void launch_hvp_at(const Ctx &c, const Phys &ph, const double *x, const double *act, const T *v, T *y, T *hp,
+                   cudaStream_t s)
+{
+    const HvpIn<T> in{nullptr, x, act};
+    hvp_tile<T, HVP_CALLER>(c, ph, in, v, y, hp, s);
+    hvp_fin<T>(c, ph, in, v, y, hp, s);
 }
 
 template <typename T>
 void launch_hvp_cg(const Ctx &c, const Phys &ph, const T *u, const T *v, T *y, T *hp, cudaStream_t s)
 {
-    hvp_tile<T, true>(c, ph, u, v, y, hp, s);
+    hvp_tile<T, HVP_CG>(c, ph, HvpIn<T>{u, nullptr, eact<T>(c)}, v, y, hp, s);
 }
 
 template <typename T>
 void launch_hvp_tile_only(const Ctx &c, const Phys &ph, const T *u, const T *v, T *y, T *hp, cudaStream_t s)
 {
-    hvp_tile<T, false>(c, ph, u, v, y, hp, s);
+    hvp_tile<T, HVP_STATE>(c, ph, HvpIn<T>{u, nullptr, eact<T>(c)}, v, y, hp, s);
 }
 
 template <typename T>
 void launch_hvp_finalize_only(const Ctx &c, const Phys &ph, const T *u, const T *v, T *y, const T *hp,
                               cudaStream_t s)
 {
-    hvp_fin<T>(c, ph, u, v, y, hp, s);
+    hvp_fin<T>(c, ph, HvpIn<T>{u, nullptr, eact<T>(c)}, v, y, hp, s);
 }
 
 void launch_param_vjp(const Ctx &c, const Phys &ph, const double *u, const double *a, const double *lam,
@@ -992,24 +1069,23 @@ cudaError_t configure_elem_kernels()
     SET((k_tile_grad<3, false>));
     SET((k_tile_grad<2, true>));
     SET((k_tile_grad<3, true>));
-#define SET_HVP(T, MB)                                                       \
-    SET((k_tile_hvp<T, 2, true, MB, 0, false>));                             \
-    SET((k_tile_hvp<T, 3, true, MB, 0, false>));                             \
-    SET((k_tile_hvp<T, 2, false, MB, 0, false>));                            \
-    SET((k_tile_hvp<T, 3, false, MB, 0, false>));                            \
-    SET((k_tile_hvp<T, 2, true, MB, 0, true>));                              \
-    SET((k_tile_hvp<T, 3, true, MB, 0, true>));                              \
-    SET((k_tile_hvp<T, 2, false, MB, 0, true>));                             \
-    SET((k_tile_hvp<T, 3, false, MB, 0, true>));                             \
-    SET((k_tile_hvp<T, 2, true, MB, (sizeof(T) == 4 ? kCap2 : 0), false>));  \
-    SET((k_tile_hvp<T, 3, true, MB, (sizeof(T) == 4 ? kCap3 : 0), false>));  \
-    SET((k_tile_hvp<T, 2, false, MB, (sizeof(T) == 4 ? kCap2 : 0), false>)); \
-    SET((k_tile_hvp<T, 3, false, MB, (sizeof(T) == 4 ? kCap3 : 0), false>));
+#define SET_MODE(T, MB, M)                                                \
+    SET((k_tile_hvp<T, 2, M, MB, 0, false>));                             \
+    SET((k_tile_hvp<T, 3, M, MB, 0, false>));                             \
+    SET((k_tile_hvp<T, 2, M, MB, 0, true>));                              \
+    SET((k_tile_hvp<T, 3, M, MB, 0, true>));                              \
+    SET((k_tile_hvp<T, 2, M, MB, (sizeof(T) == 4 ? kCap2 : 0), false>));  \
+    SET((k_tile_hvp<T, 3, M, MB, (sizeof(T) == 4 ? kCap3 : 0), false>));
+#define SET_HVP(T, MB)          \
+    SET_MODE(T, MB, HVP_STATE)  \
+    SET_MODE(T, MB, HVP_CG)     \
+    SET_MODE(T, MB, HVP_CALLER)
     SET_HVP(float, 3)
     SET_HVP(float, 4)
     SET_HVP(double, 1)
     SET_HVP(double, 2)
 #undef SET_HVP
+#undef SET_MODE
     SET((k_tile_vjp<2>));
     SET((k_tile_vjp<3>));
     SET((k_tile_mat_vjp<2>));
@@ -1022,6 +1098,10 @@ template void launch_hvp<float>(const Ctx &, const Phys &, const float *, const 
                                 cudaStream_t);
 template void launch_hvp<double>(const Ctx &, const Phys &, const double *, const double *, double *, double *,
                                  cudaStream_t);
+template void launch_hvp_at<float>(const Ctx &, const Phys &, const double *, const double *, const float *, float *,
+                                   float *, cudaStream_t);
+template void launch_hvp_at<double>(const Ctx &, const Phys &, const double *, const double *, const double *,
+                                    double *, double *, cudaStream_t);
 template void launch_hvp_cg<float>(const Ctx &, const Phys &, const float *, const float *, float *, float *,
                                    cudaStream_t);
 template void launch_hvp_cg<double>(const Ctx &, const Phys &, const double *, const double *, double *, double *,

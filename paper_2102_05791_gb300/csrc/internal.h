@@ -9,7 +9,7 @@
 //     W (1), f (dim); FP64, read by the energy, gradient and VJP kernels.
 //   * The HVP kernels read per-element records instead, [ne_int][rs] (FP32 and
 //     FP64 copies): the hvp_fields() fields in the order above (f only with
-//     the spring muscle), the activation, padding to rs = rec_stride(), and
+//     the spring muscle), a slot for the activation, padding to rs = rec_stride(), and
 //     in shared memory the element's corner forces overwrite its own record
 //     from slot corner_base(local elem).
 //   * conn[e] packs the element's dim+1 tile-local vertex ids, 8 bits each.
@@ -158,9 +158,12 @@ struct Ctx {
     VertDev vd;
     ElemDev<double> e64;
     // HVP element records [ne_int][td.rs] in tile order: the hvp_fields()
-    // element fields, then the activation (written by set_activation)
-    float *rec32 = nullptr;   // mixed precision only
-    double *rec64 = nullptr;
+    // element fields, then a free slot for the activation
+    const float *rec32 = nullptr;   // mixed precision only
+    const double *rec64 = nullptr;
+    // the call's activations in tile order (set_inputs)
+    float *a32 = nullptr;           // mixed precision only
+    double *a64 = nullptr;
     int threads = 256;
     int muscle = 0;              // muscle model (the spring's HVP also stages the fiber)
     double *partials = nullptr;  // [n_partials] FP64 block partial sums
@@ -192,6 +195,10 @@ int eval_split(int n_tiles, int sms);  // CTAs per tile of the gradient kernel
 // come from the element records.
 template <typename T>
 void launch_hvp(const Ctx &c, const Phys &ph, const T *u, const T *v, T *y, T *hp, cudaStream_t s);
+// The same with the caller's positions x and activations (caller order).
+template <typename T>
+void launch_hvp_at(const Ctx &c, const Phys &ph, const double *x, const double *act, const T *v, T *y, T *hp,
+                   cudaStream_t s);
 template <typename T>
 void launch_hvp_tile_only(const Ctx &c, const Phys &ph, const T *u, const T *v, T *y, T *hp, cudaStream_t s);
 template <typename T>
@@ -242,14 +249,14 @@ void launch_tile_dot(const Ctx &c, double *out, cudaStream_t s);
 template <typename T>
 void launch_step_update(const Ctx &c, double *u, const T *d, double t, float *u32, cudaStream_t s);
 
-void launch_x_to_u(const Ctx &c, const double *x, double *u, float *u32, const uint8_t *fixed_pin,
-                   cudaStream_t s);
 void launch_u_to_x(const Ctx &c, const double *u, double *x, cudaStream_t s);
 void launch_uhat(const Ctx &c, const double *x0, const double *v0, double dt, double *uhat,
                  cudaStream_t s);
-// The caller's activations in tile order (0 for padding elements): dense FP64,
-// and the activation slots of the FP64 and FP32 records; null: not wanted.
-void launch_set_activation(const Ctx &c, const double *user, double *a64, double *r64, float *r32, cudaStream_t s);
+// A call's inputs in the library's own form: displacements u = x - X (0 at
+// pinned vertices when `fixed` is given) and activations in tile order (0 for
+// padding elements), FP64 and FP32; null outputs are skipped.
+void launch_set_inputs(const Ctx &c, const double *x, double *u, float *u32, const uint8_t *fixed, const double *a,
+                       double *a64, float *a32, cudaStream_t s);
 template <typename Tin, typename Tout>
 void launch_convert(int64_t n, const Tin *in, Tout *out, cudaStream_t s);
 void launch_mask_copy(const Ctx &c, const double *in, double *out, cudaStream_t s);

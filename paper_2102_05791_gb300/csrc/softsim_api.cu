@@ -44,7 +44,7 @@ struct WhileGraph {
 }  // namespace
 
 struct sim_handle {
-    int dim = 0, precision = SIM_PREC_MIXED, device = 0;
+    int dim = 0, precision = SIM_PREC_MIXED, device = 0, n_sm = 0;
     int64_t nv = 0, ne = 0;
     sim_material mat{};
     sim_options opt{};
@@ -54,7 +54,7 @@ struct sim_handle {
     // device state
     double *X = nullptr, *mass = nullptr;
     uint8_t *fixed = nullptr;
-    double *u = nullptr, *uhat = nullptr, *g = nullptr, *hp64 = nullptr, *a64 = nullptr;
+    double *u = nullptr, *uhat = nullptr, *g = nullptr, *hp64 = nullptr;
     double *fw = nullptr, *u0 = nullptr;  // ground friction of the current step (null when off)
     float *u32 = nullptr, *hp32 = nullptr;
     float *u4 = nullptr;  // 3D FP32 displacement in 16-byte rows, as the CG tile kernel gathers it
@@ -375,18 +375,18 @@ static int create_impl(sim_handle *h, const sim_mesh *mesh, const sim_material *
     c.e64.base = ce64;
     c.e64.stride = ne_int;
     {
-        // HVP records: the first nf_hvp fields in the FI order, activation slot and padding zero
+        // HVP records: the first nf_hvp fields in the FI order, the rest zero
         std::vector<double> rec((size_t)rs * ne_int, 0.0);
         for (int64_t i = 0; i < ne_int; ++i)
             for (int f = 0; f < nf_hvp; ++f) rec[(size_t)i * rs + f] = edata[(size_t)f * ne_int + i];
         const double *cr64;
         if ((rc = upload(h, rec, &cr64))) return rc;
-        c.rec64 = const_cast<double *>(cr64);
+        c.rec64 = cr64;
         if (is_mixed(h)) {
             std::vector<float> rec32(rec.begin(), rec.end());
             const float *cr32;
             if ((rc = upload(h, rec32, &cr32))) return rc;
-            c.rec32 = const_cast<float *>(cr32);
+            c.rec32 = cr32;
         }
     }
     c.vd.nv = nv;
@@ -446,9 +446,8 @@ static int create_impl(sim_handle *h, const sim_mesh *mesh, const sim_material *
     c.muscle = h->mat.muscle_model;
     if (c.threads % 32 || c.threads > 256) return fail(h, SIM_EINVAL, "threads must be a multiple of 32, at most 256");
     c.n_fin_blocks = std::max(1, (td.n_fin + 255) / 256);
-    int n_sm = 0;
-    CK(h, cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, h->device));
-    c.split = eval_split(td.n_tiles, n_sm);
+    CK(h, cudaDeviceGetAttribute(&h->n_sm, cudaDevAttrMultiProcessorCount, h->device));
+    c.split = eval_split(td.n_tiles, h->n_sm);
 
     // --- work buffers
     const int64_t nd = nv * d;
@@ -467,7 +466,8 @@ static int create_impl(sim_handle *h, const sim_mesh *mesh, const sim_material *
     h->r64 = (double *)dalloc(h, sizeof(double) * nd);
     h->Hx = (double *)dalloc(h, sizeof(double) * nd);
     h->hp64 = (double *)dalloc(h, sizeof(double) * std::max<int64_t>(tb.n_slots, 1) * d);
-    h->a64 = (double *)dalloc(h, sizeof(double) * ne_int);
+    c.a64 = (double *)dalloc(h, sizeof(double) * ne_int);
+    if (is_mixed(h)) c.a32 = (float *)dalloc(h, sizeof(float) * ne_int);
     h->vd = dalloc(h, vbytes * nd);
     h->vr = dalloc(h, vbytes * nd);
     h->vp = dalloc(h, vbytes * nd);
@@ -480,7 +480,7 @@ static int create_impl(sim_handle *h, const sim_mesh *mesh, const sim_material *
             if (!h->u4) return fail(h, SIM_ENOMEM, "device allocation failed");
         }
     }
-    if (!c.partials || !h->sc || !h->u || !h->uhat || !h->g || !h->work || !h->lam || !h->lacc || !h->r64 || !h->Hx || !h->hp64 || !h->a64 || !h->vd ||
+    if (!c.partials || !h->sc || !h->u || !h->uhat || !h->g || !h->work || !h->lam || !h->lacc || !h->r64 || !h->Hx || !h->hp64 || !c.a64 || (is_mixed(h) && !c.a32) || !h->vd ||
         !h->vr || !h->vp || !h->vAp || (is_mixed(h) && (!h->u32 || !h->hp32)))
         return fail(h, SIM_ENOMEM, "device allocation failed");
     CK(h, cudaMemset(h->sc, 0, sizeof(DevScalars)));
@@ -560,26 +560,15 @@ struct View<double> {
     static double *hp(sim_handle *h) { return h->hp64; }
 };
 
-// The copies of the caller's activations a call reads.  A record's slot is 4
-// or 8 bytes of a record of its own sectors (31 us each at 3.1 million tets),
-// so only what is read is written.
-enum { ACT_DENSE = 1, ACT_REC = 2, ACT_REC64 = 4 };  // FP64 array; records of the handle's precision; FP64 records
-
-static int set_activation(sim_handle *h, const double *a, int what, cudaStream_t s)
+// Set the internal displacement and activations from the caller's positions
+// and activations; pin = clamp pinned vertices to rest.  FP64 = false: only the
+// copies of the handle's own precision are wanted.
+static int set_inputs(sim_handle *h, const double *x, bool pin, const double *a, bool fp64, cudaStream_t s)
 {
-    const Ctx &c = h->ctx;
-    const int slot = hvp_fields(c.dim, c.muscle == SIM_MUSCLE_SPRING);  // after the HVP fields
-    const bool r64 = (what & ACT_REC64) || (!is_mixed(h) && (what & ACT_REC)), r32 = is_mixed(h) && (what & ACT_REC);
-    launch_set_activation(c, a, what & ACT_DENSE ? h->a64 : nullptr, r64 ? c.rec64 + slot : nullptr,
-                          r32 ? c.rec32 + slot : nullptr, s);
-    CKL(h);
-    return SIM_OK;
-}
-
-// Set the internal displacement from positions; pin = clamp pinned vertices to rest.
-static int set_state(sim_handle *h, const double *x, bool pin, cudaStream_t s)
-{
-    launch_x_to_u(h->ctx, x, h->u, h->u32, pin ? h->fixed : nullptr, s);
+    Ctx &c = h->ctx;
+    fp64 = fp64 || !is_mixed(h);
+    launch_set_inputs(c, x, fp64 ? h->u : nullptr, h->u32, pin ? h->fixed : nullptr, a, fp64 ? c.a64 : nullptr, c.a32,
+                      s);
     CKL(h);
     return SIM_OK;
 }
@@ -730,9 +719,8 @@ static PcgSizes pcg_sizes(int dim, bool f32, int64_t nv, int n_sm)
 template <typename T>
 static int build_pcg(sim_handle *h)
 {
-    int n_sm = 0, rc;
-    CK(h, cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, h->device));
-    const PcgSizes z = pcg_sizes(h->dim, sizeof(T) == 4, h->nv, n_sm);
+    int rc;
+    const PcgSizes z = pcg_sizes(h->dim, sizeof(T) == 4, h->nv, h->n_sm);
     CgPlan P;
     std::string err;
     h->pcg_state = -1;
@@ -853,7 +841,7 @@ static int newton_impl(sim_handle *h, bool dyn, sim_solve_stats *st, cudaStream_
     const double *uh = dyn ? h->uhat : nullptr;
     const double t0 = 0.0;
     double *u_prev = h->Hx;  // the state before the step (FP64 vector of the adjoint, unused here)
-    launch_grad(c, ph, h->u, uh, h->a64, h->g, h->hp64, true, s);
+    launch_grad(c, ph, h->u, uh, c.a64, h->g, h->hp64, true, s);
     CKL(h);
     if ((rc = read_scalars(h, s))) return rc;
     double gn = std::sqrt(h->sc_host->gn2);
@@ -890,7 +878,7 @@ static int newton_impl(sim_handle *h, bool dyn, sim_solve_stats *st, cudaStream_
         // line search: t = 1, taken and evaluated in full (energy and gradient
         // share their work); on rejection undone, then batches of halvings
         launch_newton_step<T>(c, h->g, (const T *)h->vd, h->u, u_prev, h->u32, s);
-        launch_grad(c, ph, h->u, uh, h->a64, h->g, h->hp64, true, s);
+        launch_grad(c, ph, h->u, uh, c.a64, h->g, h->hp64, true, s);
         CKL(h);
         if ((rc = read_scalars(h, s))) return rc;
         S.cg_iters_total += h->sc_host->iter;
@@ -914,7 +902,7 @@ static int newton_impl(sim_handle *h, bool dyn, sim_solve_stats *st, cudaStream_
         if (!ok) {
             CK(h, cudaMemcpyAsync(h->u, u_prev, sizeof(double) * c.nv * c.dim, cudaMemcpyDeviceToDevice, s));
             if (fix) {  // no descent direction: d := -g
-                launch_grad(c, ph, h->u, uh, h->a64, h->g, h->hp64, false, s);
+                launch_grad(c, ph, h->u, uh, c.a64, h->g, h->hp64, false, s);
                 launch_dir_check<T>(c, h->g, (T *)h->vd, s);
             }
             const double *dir64 = (const double *)h->vd;
@@ -928,7 +916,7 @@ static int newton_impl(sim_handle *h, bool dyn, sim_solve_stats *st, cudaStream_
                 const int nt = j0 == 0 ? 1 : std::min(kMaxTrials, h->opt.max_ls - j0);
                 double ts[kMaxTrials];
                 for (int j = 0; j < nt; ++j) ts[j] = std::ldexp(1.0, -(j0 + j));
-                launch_energy(c, ph, h->u, dir64, uh, h->a64, ts, nt, s);
+                launch_energy(c, ph, h->u, dir64, uh, c.a64, ts, nt, s);
                 CKL(h);
                 if ((rc = read_scalars(h, s))) return rc;
                 for (int j = 0; j < nt && !ok; ++j) ok = accept(j0 + j, ts[j], j);
@@ -936,7 +924,7 @@ static int newton_impl(sim_handle *h, bool dyn, sim_solve_stats *st, cudaStream_
             }
             if (ok) {
                 launch_step_update<T>(c, h->u, (const T *)h->vd, t_acc, h->u32, s);
-                launch_grad(c, ph, h->u, uh, h->a64, h->g, h->hp64, true, s);
+                launch_grad(c, ph, h->u, uh, c.a64, h->g, h->hp64, true, s);
                 CKL(h);
                 if ((rc = read_scalars(h, s))) return rc;
             }
@@ -946,7 +934,7 @@ static int newton_impl(sim_handle *h, bool dyn, sim_solve_stats *st, cudaStream_
             S.ls_halvings += h->opt.max_ls;
             S.status = SIM_ELINESEARCH;
             // the smallest J of the state that stays
-            launch_energy(c, ph, h->u, nullptr, uh, h->a64, &t0, 1, s);
+            launch_energy(c, ph, h->u, nullptr, uh, c.a64, &t0, 1, s);
             CKL(h);
             if ((rc = read_scalars(h, s))) return rc;
             break;
@@ -1068,13 +1056,12 @@ extern "C" int sim_energy_grad(sim_handle *h, const double *x, const double *a, 
     if (!x || !a) return fail(h, SIM_EINVAL, "null x or a");
     cudaStream_t s = (cudaStream_t)stream;
     int rc;
-    if ((rc = set_state(h, x, false, s))) return rc;
-    if ((rc = set_activation(h, a, ACT_DENSE, s))) return rc;
+    if ((rc = set_inputs(h, x, false, a, true, s))) return rc;
     const Phys ph = make_phys(h, false);
-    if (grad) launch_grad(h->ctx, ph, h->u, nullptr, h->a64, grad, h->hp64, E_dev != nullptr, s);
+    if (grad) launch_grad(h->ctx, ph, h->u, nullptr, h->ctx.a64, grad, h->hp64, E_dev != nullptr, s);
     if (E_dev) {
         const double t0 = 0.0;
-        if (!grad) launch_energy(h->ctx, ph, h->u, nullptr, nullptr, h->a64, &t0, 1, s);
+        if (!grad) launch_energy(h->ctx, ph, h->u, nullptr, nullptr, h->ctx.a64, &t0, 1, s);
         CK(h, cudaMemcpyAsync(E_dev, &h->sc->E[0], sizeof(double), cudaMemcpyDeviceToDevice, s));
     }
     CKL(h);
@@ -1086,10 +1073,22 @@ extern "C" int sim_hvp(sim_handle *h, const double *x, const double *a, const vo
     CHECK_H(h);
     if (!x || !a || !v || !Hv) return fail(h, SIM_EINVAL, "null argument");
     cudaStream_t s = (cudaStream_t)stream;
-    int rc;
-    if ((rc = set_state(h, x, false, s))) return rc;
-    if ((rc = set_activation(h, a, ACT_REC, s))) return rc;
     const Phys ph = make_phys(h, false);
+    // One wave of tiles or less: the tile kernel converts x and a itself, which
+    // costs it less than a launch (1,122 triangles: 22.0 us the call, 23.8 with
+    // the conversions in launches of their own).  With many waves every tile
+    // pays for the scattered FP64 reads (3.1 million tets: 99 us against 58 + 19
+    // with them converted first).
+    if (h->ctx.td.n_tiles <= h->n_sm) {
+        if (is_mixed(h))
+            launch_hvp_at<float>(h->ctx, ph, x, a, (const float *)v, (float *)Hv, h->hp32, s);
+        else
+            launch_hvp_at<double>(h->ctx, ph, x, a, (const double *)v, (double *)Hv, h->hp64, s);
+        CKL(h);
+        return SIM_OK;
+    }
+    int rc;
+    if ((rc = set_inputs(h, x, false, a, false, s))) return rc;
     if (is_mixed(h))
         launch_hvp<float>(h->ctx, ph, h->u32, (const float *)v, (float *)Hv, h->hp32, s);
     else
@@ -1126,8 +1125,7 @@ extern "C" int sim_hvp_dot(sim_handle *h, const double *x, const double *a, cons
     if (!x || !a || !v || !Hv || !vHv) return fail(h, SIM_EINVAL, "null argument");
     cudaStream_t s = (cudaStream_t)stream;
     int rc;
-    if ((rc = set_state(h, x, false, s))) return rc;
-    if ((rc = set_activation(h, a, ACT_REC, s))) return rc;
+    if ((rc = set_inputs(h, x, false, a, true, s))) return rc;
     return is_mixed(h) ? hvp_dot_impl<float>(h, v, Hv, vHv, s) : hvp_dot_impl<double>(h, v, Hv, vHv, s);
 }
 
@@ -1143,10 +1141,9 @@ extern "C" int sim_newton_solve(sim_handle *h, const double *x_init, const doubl
     if (!x_init) return fail(h, SIM_EINVAL, "null x_init");
     cudaStream_t s = (cudaStream_t)stream;
     int rc;
-    if ((rc = set_activation(h, a, ACT_DENSE | ACT_REC, s))) return rc;
     if (dyn) launch_uhat(h->ctx, x0, v0, h->mat.dt, h->uhat, s);
     if (dyn && h->fw) launch_friction_prep(h->ctx, x0, h->mat.k_friction, h->mat.eps_friction, h->u0, h->fw, s);
-    if ((rc = set_state(h, x_init, true, s))) return rc;
+    if ((rc = set_inputs(h, x_init, true, a, true, s))) return rc;
     const int status = is_mixed(h) ? newton_impl<float>(h, dyn, st, s) : newton_impl<double>(h, dyn, st, s);
     if (status == SIM_ECUDA) return status;
     launch_u_to_x(h->ctx, h->u, x_out, s);
@@ -1163,8 +1160,7 @@ extern "C" int sim_adjoint_solve(sim_handle *h, const double *x_star, const doub
     if (!x_star || !a || !dLdx || !lambda) return fail(h, SIM_EINVAL, "null argument");
     cudaStream_t s = (cudaStream_t)stream;
     int rc;
-    if ((rc = set_state(h, x_star, false, s))) return rc;
-    if ((rc = set_activation(h, a, ACT_REC | ACT_REC64, s))) return rc;
+    if ((rc = set_inputs(h, x_star, false, a, true, s))) return rc;
     const bool dyn = h->mat.dt > 0.0;
     const int status = is_mixed(h) ? adjoint_impl<float>(h, dyn, dLdx, lambda, st, s)
                                    : adjoint_impl<double>(h, dyn, dLdx, lambda, st, s);
@@ -1181,10 +1177,9 @@ extern "C" int sim_param_vjp(sim_handle *h, const double *x_star, const double *
     if (!x_star || !a || !lambda || !dLda) return fail(h, SIM_EINVAL, "null argument");
     cudaStream_t s = (cudaStream_t)stream;
     int rc;
-    if ((rc = set_state(h, x_star, false, s))) return rc;
-    if ((rc = set_activation(h, a, ACT_DENSE, s))) return rc;
+    if ((rc = set_inputs(h, x_star, false, a, true, s))) return rc;
     const Phys ph = make_phys(h, h->mat.dt > 0.0);
-    launch_param_vjp(h->ctx, ph, h->u, h->a64, lambda, dLda, s);
+    launch_param_vjp(h->ctx, ph, h->u, h->ctx.a64, lambda, dLda, s);
     CKL(h);
     return SIM_OK;
 }
@@ -1197,10 +1192,9 @@ extern "C" int sim_material_vjp(sim_handle *h, const double *x_star, const doubl
     if (!dLdmu && !dLdlambda && !dLdk) return SIM_OK;
     cudaStream_t s = (cudaStream_t)stream;
     int rc;
-    if ((rc = set_state(h, x_star, false, s))) return rc;
-    if ((rc = set_activation(h, a, ACT_DENSE, s))) return rc;
+    if ((rc = set_inputs(h, x_star, false, a, true, s))) return rc;
     const Phys ph = make_phys(h, h->mat.dt > 0.0);
-    launch_material_vjp(h->ctx, ph, h->u, h->a64, lambda, dLdmu, dLdlambda, dLdk, s);
+    launch_material_vjp(h->ctx, ph, h->u, h->ctx.a64, lambda, dLdmu, dLdlambda, dLdk, s);
     CKL(h);
     return SIM_OK;
 }

@@ -58,3 +58,27 @@ def test_rejected_full_steps(dims, precision, stretch):
     assert np.linalg.norm(m.grad(host(x), p.a)) <= 1.01e-9 * g0
     assert abs(st["min_J"] - m.min_J(host(x))) <= 1e-12
     sim.close()
+
+
+@pytest.mark.parametrize("dims,precision,muscle", [
+    ((1, 1), "mixed", 0), ((33, 17), "fp64", 1), ((41, 25), "mixed", 1), ((300, 140), "mixed", 0),
+    ((1, 1, 1), "fp64", 0), ((11, 7, 9), "mixed", 1), ((24, 21, 20), "mixed", 0), ((24, 21, 20), "fp64", 1)])
+def test_hvp_from_the_callers_arrays(dims, precision, muscle):
+    """One wave of tiles or less converts x and a in the tile kernel, more tiles in a pass before it.  Against the
+    oracle: FP64 as the gradient above; FP32 inputs rounded to 6e-8, amplified by the same cancellation (a few hundred
+    times at most in the norm): 2e-5.  Random element order."""
+    p = _make(dims)
+    p.muscle_model = muscle
+    p.k_contact, p.contact_power = 1e5, 3
+    order = np.random.default_rng(404).permutation(p.n_elem)
+    p.T, p.fiber, p.a = p.T[order], p.fiber[order], np.random.default_rng(405).uniform(0.3, 0.9, p.n_elem)
+    m = oracle.make_model(p)
+    x = deformed(p, min(0.02, 0.2 / dims[1]), seed=406)
+    v = np.random.default_rng(407).standard_normal(x.shape)
+    v[p.fixed.astype(bool)] = 0.0
+    sim = make_sim(p, precision, muscle_model=muscle)
+    y = host(sim.hvp(dev(x), dev(p.a), dev(v, sim.vec_dtype)))
+    ref = m.hvp(x, p.a, v)
+    tol = 1e-12 if precision == "fp64" else 2e-5
+    assert np.linalg.norm(y - ref) <= tol * np.linalg.norm(ref)
+    sim.close()
