@@ -530,7 +530,9 @@ __device__ __noinline__ void assemble(const BatchDev &b, const Mesh &m, Team &tm
         load_elem<float, D>(b.e32, b.estride, e, B, gv, W, f);
         edge_of<float, float, D>(b.u32, m, lid, Du);
         elem_blocks<float, D>(B, gv, f, W * b.dt2_f, b.a32[e], Du, b.muscle != 0, b.log_mode, m.mu_f, m.lam_f, b.k_f,
-                              pd.cpos + (int64_t)le * NP, contrib);
+                              [&](int pair, const float K[D][D]) {
+                                  store_block<float, D>(contrib, pd.cpos[(int64_t)le * NP + pair], K);
+                              });
     }
     {
         VertDev vd;

@@ -10,12 +10,27 @@
 
 namespace softsim {
 
-// Blocks of the element's corner pairs into their contribution slots cpos
-// (+ 2D: 3, 3D: 6 of them); W is scaled, f is used by the spring muscle only.
+// A pair's block K into its contribution slot (w: slot | kCgTransposed).
 template <typename T, int D>
+__device__ __forceinline__ void store_block(T *contrib, uint32_t w, const T K[D][D])
+{
+    T *out = contrib + (int64_t)(w & ~kCgTransposed) * (D * D);
+    const bool tr = (w & kCgTransposed) != 0;
+    if constexpr (sizeof(T) == 4 && D == 2) {
+        *reinterpret_cast<float4 *>(out) = make_float4(K[0][0], tr ? K[1][0] : K[0][1], tr ? K[0][1] : K[1][0], K[1][1]);
+        return;
+    }
+#pragma unroll
+    for (int i = 0; i < D; ++i)
+#pragma unroll
+        for (int j = 0; j < D; ++j) out[i * D + j] = tr ? K[j][i] : K[i][j];
+}
+
+// Blocks of the element's corner pairs (2D: 3, 3D: 6), each to emit(pair, K); W
+// is scaled, f is used by the spring muscle only.
+template <typename T, int D, typename Emit>
 __device__ __forceinline__ void elem_blocks(const T B[D][D], const T gv[D], const T f[D], T W, T aval, const T Du[D][D],
-                                            bool spring, int log_mode, T mu, T lam, T kk, const uint32_t *cpos,
-                                            T *contrib)
+                                            bool spring, int log_mode, T mu, T lam, T kk, Emit emit)
 {
     T F[D][D], C[D][D];
     mul<T, D>(Du, B, F, true);
@@ -68,7 +83,6 @@ __device__ __forceinline__ void elem_blocks(const T B[D][D], const T gv[D], cons
     for (int a = 0; a <= D; ++a)
 #pragma unroll
         for (int b = a + 1; b <= D; ++b, ++pair) {
-            const uint32_t w = cpos[pair];
             T K[D][D];
             T gg = T(0);
 #pragma unroll
@@ -106,12 +120,7 @@ __device__ __forceinline__ void elem_blocks(const T B[D][D], const T gv[D], cons
 #pragma unroll
                     for (int j = 0; j < D; ++j) K[i][j] += m * q[i] * q[j];
             }
-            T *out = contrib + (int64_t)(w & ~kCgTransposed) * (D * D);
-            const bool tr = (w & kCgTransposed) != 0;
-#pragma unroll
-            for (int i = 0; i < D; ++i)
-#pragma unroll
-                for (int j = 0; j < D; ++j) out[i * D + j] = tr ? K[j][i] : K[i][j];
+            emit(pair, K);
         }
 }
 

@@ -168,6 +168,7 @@ struct Ctx {
     int muscle = 0;              // muscle model (the spring's HVP also stages the fiber)
     double *partials = nullptr;  // [n_partials] FP64 block partial sums
     int n_fin_blocks = 1;
+    int asm_split = 1;           // CTAs per tile of the assembly's element kernel
     int split = 1;               // CTAs (one cluster) per tile of the gradient kernel
     DevScalars *sc = nullptr;
     mutable int64_t n_launch = 0;  // kernels launched through this context

@@ -448,6 +448,8 @@ static int create_impl(sim_handle *h, const sim_mesh *mesh, const sim_material *
     c.n_fin_blocks = std::max(1, (td.n_fin + 255) / 256);
     CK(h, cudaDeviceGetAttribute(&h->n_sm, cudaDevAttrMultiProcessorCount, h->device));
     c.split = eval_split(td.n_tiles, h->n_sm);
+    // element kernel of the assembly: warps for every SM, one element a thread at most
+    c.asm_split = std::min((td.max_te + c.threads - 1) / c.threads, std::max(1, 8 * h->n_sm / td.n_tiles));
 
     // --- work buffers
     const int64_t nd = nv * d;
