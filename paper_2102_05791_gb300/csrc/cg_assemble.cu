@@ -11,6 +11,7 @@
 #include <cstdint>
 
 #include "cg_blocks.cuh"
+#include "pdl.cuh"
 
 namespace softsim {
 
@@ -41,6 +42,7 @@ __global__ void __launch_bounds__(256) k_asm_elem(TileDev td, const T *__restric
         for (int c = 0; c < D; ++c) su[k * D + c] = u[gid * D + c];
     }
     __syncthreads();
+    pdl_trigger();
     const T mu = pick<T>(ph.mu, ph.mu_f), lam = pick<T>(ph.lam, ph.lam_f);
     const T sel = pick<T>(ph.s_el, ph.s_el_f), kk = pick<T>(ph.k, ph.k_f);
     for (int l0 = (blockIdx.y * (blockDim.x >> 5) + wrp) * 32; l0 < ne_t; l0 += gridDim.y * blockDim.x) {
@@ -91,11 +93,14 @@ __global__ void __launch_bounds__(256) k_asm_edge(int64_t n_edges, const int32_t
                                                   const T *__restrict__ contrib, T *__restrict__ blk)
 {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int q0 = e < n_edges ? edge_ptr[e] : 0, q1 = e < n_edges ? edge_ptr[e + 1] : 0;
+    pdl_trigger();
+    pdl_wait();
     if (e >= n_edges) return;
     T acc[D * D];
 #pragma unroll
     for (int k = 0; k < D * D; ++k) acc[k] = T(0);
-    for (int q = edge_ptr[e]; q < edge_ptr[e + 1]; ++q)
+    for (int q = q0; q < q1; ++q)
 #pragma unroll
         for (int k = 0; k < D * D; ++k) acc[k] += contrib[(int64_t)q * (D * D) + k];
 #pragma unroll
@@ -113,6 +118,8 @@ __global__ void __launch_bounds__(256) k_asm_slice(int64_t n_edges, const int32_
     unsigned char *base = slices + (size_t)e0 * (4 + D * D * sizeof(T));
     uint32_t *idx = reinterpret_cast<uint32_t *>(base);
     T *val = reinterpret_cast<T *>(base + (size_t)n * 4);
+    pdl_trigger();
+    pdl_wait();
     for (int k = blockIdx.y * blockDim.x + threadIdx.x; k < n; k += gridDim.y * blockDim.x) {
         const uint32_t w = ent_edge[e0 + k];
         idx[k] = ent_idx[e0 + k];
@@ -132,6 +139,7 @@ template <typename T, int D>
 __global__ void __launch_bounds__(256) k_asm_slots(PcgDev pd, VertDev vd, Phys ph, const double *__restrict__ u)
 {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait();
     if (k < pd.n_cta * pd.ns) slot_data<T, D>(k, pd, vd, ph, u);
 }
 
@@ -258,12 +266,13 @@ static void assemble(const Ctx &c, const PcgDev &pd, const Phys &ph, const T *u,
         k_asm_elem<T, D, true><<<ge, c.threads, sm, s>>>(c.td, er, ac, ph, u, pd.cpos, contrib);
     else
         k_asm_elem<T, D, false><<<ge, c.threads, sm, s>>>(c.td, er, ac, ph, u, pd.cpos, contrib);
-    k_asm_edge<T, D><<<(unsigned)((pd.n_edges + 255) / 256), 256, 0, s>>>(pd.n_edges, pd.edge_ptr, contrib, blk);
+    launch_k(true, k_asm_edge<T, D>, dim3((unsigned)((pd.n_edges + 255) / 256)), dim3(256), 0, s, pd.n_edges,
+             pd.edge_ptr, (const T *)contrib, blk);
     const dim3 gs((unsigned)pd.n_chunks, pd.tpr ? (unsigned)((pd.max_entries + 255) / 256) : 1u);
-    k_asm_slice<T, D><<<gs, 256, 0, s>>>(pd.n_edges, pd.chunk_ent, pd.ent_idx, pd.ent_edge, blk,
-                                                           pd.slices);
+    launch_k(true, k_asm_slice<T, D>, gs, dim3(256), 0, s, pd.n_edges, pd.chunk_ent, pd.ent_idx, pd.ent_edge,
+             (const T *)blk, pd.slices);
     const int n = pd.n_cta * pd.ns;
-    k_asm_slots<T, D><<<(n + 255) / 256, 256, 0, s>>>(pd, c.vd, ph, u64);
+    launch_k(true, k_asm_slots<T, D>, dim3((n + 255) / 256), dim3(256), 0, s, pd, c.vd, ph, u64);
     c.n_launch += 4;
     if (!coarse) return;
     cudaMemsetAsync(pd.E, 0, sizeof(float) * pd.n_coarse * pd.n_coarse, s);

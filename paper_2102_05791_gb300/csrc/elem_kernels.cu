@@ -280,6 +280,7 @@ __global__ void __launch_bounds__(256) k_tile_grad(TileDev td, ElemDev<double> e
     // this CTA's share of the tile's elements and of its vertices
     const int ech = (ne_t + split - 1) / split, vch = (nlv + split - 1) / split;
     const int e0 = rank * ech, e1 = min(ne_t, e0 + ech), k0 = rank * vch, k1 = min(nlv, k0 + vch);
+    pdl_wait();  // everything above is static
     for (int k = threadIdx.x; k < nlv; k += blockDim.x) {
         const int64_t gid = td.lv_gid[vs + k];
 #pragma unroll

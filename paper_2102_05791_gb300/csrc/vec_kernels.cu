@@ -266,6 +266,8 @@ __global__ void __launch_bounds__(256) k_newton_step(int64_t n, const double *__
                                                      float *__restrict__ u32, double *__restrict__ partials,
                                                      DevScalars *sc)
 {
+    pdl_trigger();
+    pdl_wait();
     double gd = 0.0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const double di = (double)d[i], u0 = u[i], ui = u0 + di;
@@ -546,7 +548,7 @@ void launch_newton_step(const Ctx &c, const double *g, const T *d, double *u, do
 {
     c.n_launch += 1;
     const int64_t n = c.nv * c.dim;
-    k_newton_step<T><<<vec_grid(n), 256, 0, s>>>(n, g, d, u, up, u32, c.partials, c.sc);
+    launch_k(true, k_newton_step<T>, dim3(vec_grid(n)), dim3(256), 0, s, n, g, d, u, up, u32, c.partials, c.sc);
 }
 
 template <typename T>
