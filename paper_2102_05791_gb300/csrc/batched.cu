@@ -131,17 +131,20 @@ struct Share {
 
 // A mesh's rollout is one serial chain, so the largest meshes decide when they
 // are few or uneven, and small ones waste the CTAs of a team.  The end of the
-// launch is modelled from a step's cost, in microseconds (measured at 120, 648
-// and 4,095 vertices on teams of 1, 2 and 4), for every team size and a few
-// sizes of n_big; meshes above per_cta vertices a CTA have no assembled CG.
-static Share share_out(const std::vector<int64_t> &nv_sorted, const int n_teams[5], int sms, int64_t per_cta)
+// launch is modelled from a step's cost, in microseconds (measured at 120 to
+// 4,140 vertices on teams of 1, 2 and 4), for every team size and a few sizes of
+// n_big.  More than four vertices a thread cost a CG iteration 26 us at 2,070
+// vertices a CTA, where four cost 15 at 1,900 (256 bodies of 200 to 8,000
+// triangles: 66.7 ms with the iteration taken as linear, 63.5 like this);
+// meshes above eight have no assembled CG.
+static Share share_out(const std::vector<int64_t> &nv_sorted, const int n_teams[5], int sms, int threads)
 {
     const int M = (int)nv_sorted.size();
     auto cost = [&](int64_t nv, int c) {
         const double v = (double)nv / c;
         const double its = 110.0 + (c == 1 ? 0.125 : 0.082) * (double)nv;
-        const double it = c == 1 ? 4.3 + 6.4e-3 * v : 4.9 + 5.0e-3 * v;
-        return (its * it + 270.0 + 1.6 * v) * (v > (double)per_cta ? 10.0 : 1.0);
+        const double it = v > 4.0 * threads - 64.0 ? 21.5 + 2.25e-3 * v : c == 1 ? 4.3 + 6.4e-3 * v : 4.9 + 5.0e-3 * v;
+        return (its * it + 270.0 + 1.6 * v) * (v > (double)kBatchVpt * threads - 256.0 ? 10.0 : 1.0);
     };
     Share best;
     double best_t = INFINITY;
@@ -209,7 +212,7 @@ static int build_plans(sim_batch *bt, const sim_mesh *meshes, const std::vector<
         nv_sorted[k] = nv[order[k]];
         place[order[k]] = k;
     }
-    const Share share = share_out(nv_sorted, n_teams, sms, (int64_t)kBatchVpt * bt->threads - 256);  // slots are padded
+    const Share share = share_out(nv_sorted, n_teams, sms, bt->threads);
     b.team = share.team;
     b.n_big = share.n_big;
     std::vector<CgPlan> plans(M);

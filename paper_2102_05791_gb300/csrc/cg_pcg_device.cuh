@@ -399,7 +399,12 @@ __device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int ct
     constexpr int NM = D == 3 ? 6 : 3, ND = D == 3 ? 6 : 3, DD = D * D, RN = Row<T, D>::N;
     constexpr int NI = (NM + 1) / 2;       // pairs of words that hold a CTA's items
     constexpr bool F32 = sizeof(T) == 4;
-    constexpr bool KEEP_Z = VPT <= 2;  // D^-1 r stays in registers between the phases
+    // A slot's arm, vertex diagonal and inverse block stay in registers where one
+    // slot a thread leaves room (walker 4.54 -> 4.09 us an iteration, 70,785
+    // vertices 13.0 -> 12.5); with four slots the spills cost more than the loads
+    // (2D 20,000 vertices 7.1 -> 7.6 us)
+    constexpr bool KEEP_S = F32 && VPT == 1;
+    constexpr bool KEEP_Z = VPT <= 2;  // so does D^-1 r between the phases
     constexpr int VB = VPT < 2 ? VPT : 2;  // slots whose loads are issued together
     constexpr int PB = VPT < 4 ? 4 : 2;    // loads of an exchange in flight per thread
     __shared__ float sred[kMaxWarps * VPT][8];  // per warp, or per group of 32 slots: restriction, two dots
@@ -696,6 +701,37 @@ __device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int ct
     };
 
     T x[VPT][D], r[VPT][D], zk[KEEP_Z ? VPT : 1][D];
+    float4 Rk[KEEP_S ? VPT : 1];
+    T dk[KEEP_S ? VPT : 1][2], Sk[KEEP_S ? VPT : 1][ND];
+    if constexpr (KEEP_S)
+#pragma unroll
+        for (int m = 0; m < VPT; ++m) {
+            const int k = tid + m * nthr;
+            Rk[m] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            dk[m][0] = dk[m][1] = T(0);
+#pragma unroll
+            for (int q = 0; q < ND; ++q) Sk[m][q] = T(0);
+            if (k >= ns) continue;
+            Rk[m] = pos(k);
+            if (pd.has_diag) dk[m][0] = dg(k)[0], dk[m][1] = dg(k)[1];
+#pragma unroll
+            for (int q = 0; q < ND; ++q) Sk[m][q] = *dinv(q, k);
+        }
+    auto arm = [&](int m, int k) {
+        if constexpr (KEEP_S)
+            return Rk[m];
+        else
+            return pos(k);
+    };
+    auto inv_block = [&](int m, int k, T *S) {
+#pragma unroll
+        for (int q = 0; q < ND; ++q) {
+            if constexpr (KEEP_S)
+                S[q] = Sk[m][q];
+            else
+                S[q] = *dinv(q, k);
+        }
+    };
 #pragma unroll
     for (int m = 0; m < VPT; ++m)
 #pragma unroll
@@ -732,9 +768,8 @@ __device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int ct
             for (int c = 0; c < D; ++c) r[m][c] = T(rhs(k, c) * scale);
             if (k < ns) {
                 T S[ND];
-#pragma unroll
-                for (int q = 0; q < ND; ++q) S[q] = *dinv(q, k);
-                residual(m, k, S, pos(k), r[m], v, d_rr, d_rz);
+                inv_block(m, k, S);
+                residual(m, k, S, arm(m, k), r[m], v, d_rr, d_rz);
                 if (!one) {
                     put_sum(m, v);
 #pragma unroll
@@ -779,7 +814,7 @@ __device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int ct
             for (int u = 0; u < VB; ++u) {
                 const int k = tid + (m0 + u) * nthr;
                 if (k >= ns) continue;
-                R[u] = pos(k);
+                R[u] = arm(m0 + u, k);
                 if constexpr (KEEP_Z) {
 #pragma unroll
                     for (int c = 0; c < D; ++c) z[u][c] = zk[m0 + u][c];
@@ -855,9 +890,12 @@ __device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int ct
                 for (int u = 0; u < VB; ++u) {
                     const int k = tid + (m0 + u) * nthr;
                     if (k >= ns) continue;
-                    R[u] = pos(k);
+                    R[u] = arm(m0 + u, k);
                     dh[u] = dy[u] = T(0);
-                    if (pd.has_diag) dh[u] = dg(k)[0], dy[u] = dg(k)[1];
+                    if constexpr (KEEP_S)
+                        dh[u] = dk[m0 + u][0], dy[u] = dk[m0 + u][1];
+                    else if (pd.has_diag)
+                        dh[u] = dg(k)[0], dy[u] = dg(k)[1];
                 }
 #pragma unroll
                 for (int u = 0; u < VB; ++u) {
@@ -937,9 +975,8 @@ __device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int ct
                 for (int u = 0; u < VB; ++u) {
                     const int k = tid + (m0 + u) * nthr;
                     if (k >= ns) continue;
-                    R[u] = pos(k);
-#pragma unroll
-                    for (int q = 0; q < ND; ++q) S[u][q] = *dinv(q, k);
+                    R[u] = arm(m0 + u, k);
+                    inv_block(m0 + u, k, S[u]);
                 }
 #pragma unroll
                 for (int u = 0; u < VB; ++u) {
