@@ -515,11 +515,13 @@ struct HvpSmem {
 // per local vertex adds its corners in fixed order.
 // SPRING selects the active-spring muscle at compile time, so the
 // contractile kernel carries none of its code or its extra fields.
-// MODE: HVP_STATE reads the displacement u and the activations in tile order,
-// HVP_CG also forms p.Ap, and HVP_CALLER takes positions x and activations as
+// MODE: HVP_STATE reads the displacement u and the activations in tile order;
+// HVP_CG also forms p.Ap and, launched hundreds of times on the same
+// activations, has them in the records (launch_record_activation; a load of
+// its own cost it 62.0 against 59.8 us at 3.1 million tets); HVP_CALLER takes positions x and activations as
 // the caller has them (u = x - X rounded to T while staging), which saves a
 // small mesh one launch.  A thread fetches its elements' activations before the
-// wait for the records and puts them into its records.
+// wait for the records and puts them into its records (not HVP_CG).
 enum HvpMode { HVP_STATE, HVP_CG, HVP_CALLER };
 
 template <typename T, int D, int MODE, int MINB, int MTE, bool SPRING>
@@ -579,10 +581,12 @@ __global__ void __launch_bounds__(256, MINB) k_tile_hvp(TileDev td, const T *__r
             return static_cast<const T *>(act)[es + le];
         }
     };
+    if constexpr (!CG) {
 #pragma unroll
-    for (int j = 0; j < PRE; ++j) {
-        const int le = threadIdx.x + j * blockDim.x;
-        av[j] = le < ne_t ? activation(le) : T(0);
+        for (int j = 0; j < PRE; ++j) {
+            const int le = threadIdx.x + j * blockDim.x;
+            av[j] = le < ne_t ? activation(le) : T(0);
+        }
     }
     // the flag is read before the wait so that its load overlaps the copies
     // in flight; the previous kernel has completed, so every thread reads the
@@ -627,13 +631,14 @@ __global__ void __launch_bounds__(256, MINB) k_tile_hvp(TileDev td, const T *__r
         }
         return;
     }
-    // each thread's own elements: no barrier needed
+    if constexpr (!CG) {  // each thread's own elements: no barrier needed
 #pragma unroll
-    for (int j = 0; j < PRE; ++j) {
-        const int le = threadIdx.x + j * blockDim.x;
-        if (le < ne_t) sRec[le * RS + NF] = av[j];
+        for (int j = 0; j < PRE; ++j) {
+            const int le = threadIdx.x + j * blockDim.x;
+            if (le < ne_t) sRec[le * RS + NF] = av[j];
+        }
+        for (int le = threadIdx.x + PRE * blockDim.x; le < ne_t; le += blockDim.x) sRec[le * RS + NF] = activation(le);
     }
-    for (int le = threadIdx.x + PRE * blockDim.x; le < ne_t; le += blockDim.x) sRec[le * RS + NF] = activation(le);
     const T mu = pick<T>(ph.mu, ph.mu_f), lam = pick<T>(ph.lam, ph.lam_f);
     const T sel = pick<T>(ph.s_el, ph.s_el_f), kk = pick<T>(ph.k, ph.k_f);
     // CG: p.Ap of this tile from the element quadratic forms v_e . (H_e v_e)

@@ -159,8 +159,8 @@ struct Ctx {
     ElemDev<double> e64;
     // HVP element records [ne_int][td.rs] in tile order: the hvp_fields()
     // element fields, then a free slot for the activation
-    const float *rec32 = nullptr;   // mixed precision only
-    const double *rec64 = nullptr;
+    float *rec32 = nullptr;   // mixed precision only
+    double *rec64 = nullptr;
     // the call's activations in tile order (set_inputs)
     float *a32 = nullptr;           // mixed precision only
     double *a64 = nullptr;
@@ -272,6 +272,9 @@ void launch_step_bwd_combine(const Ctx &c, const double *lam, const double *vbar
 void launch_axpy_out(int64_t n, const double *x, const double *y, double beta, double *out,
                      cudaStream_t s);
 // u4[i] = (u[3i], u[3i+1], u[3i+2], 0) for the 3D FP32 CG tile kernel
+// The call's activations into the records' slots, as the CG tile kernel reads them.
+template <typename T>
+void launch_record_activation(const Ctx &c, cudaStream_t s);
 void launch_pad_rows4(const Ctx &c, const float *u, float *u4, cudaStream_t s);
 // blocks of the grid-stride vector kernels for n entries
 int vec_grid_size(int64_t n);

@@ -381,12 +381,12 @@ static int create_impl(sim_handle *h, const sim_mesh *mesh, const sim_material *
             for (int f = 0; f < nf_hvp; ++f) rec[(size_t)i * rs + f] = edata[(size_t)f * ne_int + i];
         const double *cr64;
         if ((rc = upload(h, rec, &cr64))) return rc;
-        c.rec64 = cr64;
+        c.rec64 = const_cast<double *>(cr64);
         if (is_mixed(h)) {
             std::vector<float> rec32(rec.begin(), rec.end());
             const float *cr32;
             if ((rc = upload(h, rec32, &cr32))) return rc;
-            c.rec32 = cr32;
+            c.rec32 = const_cast<float *>(cr32);
         }
     }
     c.vd.nv = nv;
@@ -859,6 +859,7 @@ static int newton_impl(sim_handle *h, bool dyn, sim_solve_stats *st, cudaStream_
     }
     bool pcg;
     if ((rc = use_pcg<T>(h, &pcg))) return rc;
+    if (!pcg) launch_record_activation<T>(c, s);
     const double eps = 2.220446049250313e-16;
     int it = 0;
     for (;; ++it) {
@@ -995,6 +996,7 @@ static int adjoint_impl(sim_handle *h, bool dyn, const double *b, double *lambda
     }
     bool pcg;
     if ((rc = use_pcg<T>(h, &pcg))) return rc;
+    if (!pcg) launch_record_activation<T>(c, s);
     double rn = bn;
     const double target = h->opt.adjoint_rtol * bn;
     const double inner = is_mixed(h) ? std::max(h->opt.adjoint_rtol, 1e-4) : h->opt.adjoint_rtol;
@@ -1109,6 +1111,7 @@ static int hvp_dot_impl(sim_handle *h, const void *v, void *Hv, double *vHv, cud
     CK(h, cudaMemcpyAsync(p, v, sizeof(T) * nd, cudaMemcpyDeviceToDevice, s));
     CK(h, cudaMemsetAsync(&h->sc->done, 0, sizeof(int), s));  // the CG tile kernel skips its work once CG is done
     refresh_cg_u(h, s);
+    launch_record_activation<T>(c, s);
     launch_hvp_cg<T>(c, ph, View<T>::ucg(h), p, Ap, View<T>::hp(h), s);
     launch_hvp_finalize_only<T>(c, ph, View<T>::u(h), p, Ap, View<T>::hp(h), s);
     launch_tile_dot<T>(c, &h->sc->pAp, s);

@@ -358,6 +358,13 @@ __global__ void __launch_bounds__(256) k_set_inputs(int64_t n, int dim, const do
     }
 }
 
+template <typename T>
+__global__ void k_record_activation(int64_t ne_int, const T *__restrict__ a, T *__restrict__ slot, int64_t stride)
+{
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < ne_int; e += (int64_t)gridDim.x * blockDim.x)
+        slot[e * stride] = a[e];
+}
+
 __global__ void k_u_to_x(int64_t n, const double *__restrict__ u, const double *__restrict__ X, double *__restrict__ x)
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
@@ -568,6 +575,16 @@ void launch_set_inputs(const Ctx &c, const double *x, double *u, float *u32, con
                                                                  c.td.perm, a, a64, a32);
 }
 
+template <typename T>
+void launch_record_activation(const Ctx &c, cudaStream_t s)
+{
+    c.n_launch += 1;
+    const int slot = hvp_fields(c.dim, c.muscle != 0);  // after the fields
+    T *rec = sizeof(T) == 4 ? reinterpret_cast<T *>(c.rec32) : reinterpret_cast<T *>(c.rec64);
+    const T *a = sizeof(T) == 4 ? reinterpret_cast<const T *>(c.a32) : reinterpret_cast<const T *>(c.a64);
+    k_record_activation<T><<<vec_grid(c.ne_int), 256, 0, s>>>(c.ne_int, a, rec + slot, c.td.rs);
+}
+
 void launch_u_to_x(const Ctx &c, const double *u, double *x, cudaStream_t s)
 {
     c.n_launch += 1;
@@ -644,6 +661,7 @@ int cg_update_grid_size(int64_t nv) { return cg_vert_grid(nv); }
     template void launch_cg_alpha<T>(const Ctx &, int, cudaStream_t);                                               \
     template void launch_dir_check<T>(const Ctx &, const double *, T *, cudaStream_t);                              \
     template void launch_tile_dot<T>(const Ctx &, double *, cudaStream_t);                                          \
+    template void launch_record_activation<T>(const Ctx &, cudaStream_t);                                           \
     template void launch_newton_step<T>(const Ctx &, const double *, const T *, double *, double *, float *,        \
                                         cudaStream_t);                                                              \
     template void launch_step_update<T>(const Ctx &, double *, const T *, double, float *, cudaStream_t);           \
