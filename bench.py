@@ -10,11 +10,17 @@ min-y face pinned, gravity on; seeded synthetic inputs.
 
 Printed JSON line (rank 0):
   value      element-HVPs per second over whole steps (n_elem x CG iterations
-             of the forward and adjoint solves, divided by the step time);
+             of the forward and adjoint solves, divided by the step time; an
+             iteration applies the Hessian of all elements once, in the
+             persistent solver as one 3 x 3 block per mesh edge).  The
+             preconditioned solver needs fewer iterations for the same step,
+             so ms_per_step and solves_per_s are the figures to compare;
   e2e        the same through the public API with host buffers, including the
              host<->device copies of every step's inputs and outputs;
-  roofline   the HVP tile kernel: algorithmic bytes per launch (72 B per tet +
-             36 B per vertex) / its mean duration, against the HBM peak;
+  roofline   the HVP tile kernel (element-level HVP calls and the per-iteration
+             CG path; the timed steps' CG runs in the persistent solver):
+             algorithmic bytes per launch (72 B per tet + 36 B per vertex) / its
+             mean duration in one solve on that path, against the HBM peak;
   accuracy   the GPU results against the FP64 oracle's own stored solutions
              (tests/golden): the large body at 1/8 size and the config-3 box
              in both precisions, three bodies of the batch, the 200-step
@@ -693,7 +699,8 @@ def run_ours(args, rank, world, local_rank):
                 "traffic": recorded_traffic(args.workload, sim.tile_shape), "kernel": "k_tile_hvp<float,3>",
                 "peak_source": peak_kind}
     roof.update({"kernel_ms": tile_ms, "kernel_launches_timed": tile_n,
-                 "kernel_timing": "CUDA event nodes around every tile launch in one profiled solve after the timed steps",
+                 "kernel_timing": "CUDA event nodes around every tile launch in one profiled solve after the timed steps, on the "
+                                  "per-iteration CG path",
                  "kernel_ms_back_to_back": b2b_ms})
     line = {
         "metric": "element-HVP/s (fwd Newton-CG + adjoint, whole step)",
