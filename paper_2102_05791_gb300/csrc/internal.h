@@ -192,8 +192,8 @@ void launch_grad(const Ctx &c, const Phys &ph, const double *u, const double *uh
                  const double *a, double *g, double *hp, bool energy, cudaStream_t s);
 int eval_split(int n_tiles, int sms);  // CTAs per tile of the gradient kernel
 
-// HVP y = A v (A = H, or M + dt^2 H when ph.dyn), masked; the activations
-// come from the element records.
+// HVP y = A v (A = H, or M + dt^2 H when ph.dyn), masked, at the activations
+// of launch_set_inputs.
 template <typename T>
 void launch_hvp(const Ctx &c, const Phys &ph, const T *u, const T *v, T *y, T *hp, cudaStream_t s);
 // The same with the caller's positions x and activations (caller order).

@@ -690,7 +690,7 @@ static int cg_max_rounds(int max_iter) { return max_iter / kCgBody + 2; }
 // of nv vertices.  The lines lie where both sides measured alike (microseconds
 // an iteration on GB300): one cluster exchanges in about 1 us, a grid in about
 // 2 us, so a cluster's 16 CTAs serve as long as their rows stay in shared
-// memory (3D FP32: 4.6 us at 1,260 vertices; 8.3 on a grid of 64 at 9,537, where
+// memory (3D FP32: 4.7 us at 1,260 vertices; 7.9 on a grid of 64 at 9,537, where
 // 16 CTAs need 18; 2D: 7.2 at 20,000).  FP64 arithmetic is scarce, so FP64
 // spreads over more CTAs earlier (16.0 us on 64 CTAs against 18.8 on 16 at 2,640
 // vertices).  More aggregates save iterations but cost a larger inverse (192
