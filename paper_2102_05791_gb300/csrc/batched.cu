@@ -253,6 +253,8 @@ static int build_plans(sim_batch *bt, const sim_mesh *meshes, const std::vector<
     if (table_bytes) BCK(bt, cudaMemcpy(d0, host.data(), table_bytes, cudaMemcpyHostToDevice));
     b.pcg = bupload(bt, pds);
     if (!b.pcg) return bfail(bt, SIM_ENOMEM, "device allocation or upload failed");
+    // the uploads lie on the default stream, which a rollout on a non-blocking stream does not wait for
+    BCK(bt, cudaStreamSynchronize(nullptr));
     return SIM_OK;
 }
 

@@ -719,7 +719,7 @@ static PcgSizes pcg_sizes(int dim, bool f32, int64_t nv, int n_sm)
 }
 
 template <typename T>
-static int build_pcg(sim_handle *h)
+static int build_pcg(sim_handle *h, cudaStream_t s)
 {
     int rc;
     const PcgSizes z = pcg_sizes(h->dim, sizeof(T) == 4, h->nv, h->n_sm);
@@ -753,7 +753,10 @@ static int build_pcg(sim_handle *h)
     }
     std::vector<unsigned char> host(table_bytes);
     pcg_place_tables(P, pd, host.data(), static_cast<unsigned char *>(d0), 0);
-    CK(h, cudaMemcpy(d0, host.data(), table_bytes, cudaMemcpyHostToDevice));
+    // on the solve's stream, whose kernels read the tables next: a copy on the default stream is not
+    // ordered before a non-blocking stream's kernels; waited for while `host` is alive
+    CK(h, cudaMemcpyAsync(d0, host.data(), table_bytes, cudaMemcpyHostToDevice, s));
+    CK(h, cudaStreamSynchronize(s));
     pcg_place_buffers<T>(P, pd, static_cast<unsigned char *>(d1), 0);
     if (h->verbose)
         fprintf(stderr, "[softsim] persistent CG: %d CTAs%s x %d threads, %d slots, %d halo, %d coarse, %s, %d stages\n",
@@ -765,14 +768,14 @@ static int build_pcg(sim_handle *h)
 
 // Whether this handle's CG solves run as one persistent launch; builds its plan on the first call.
 template <typename T>
-static int use_pcg(sim_handle *h, bool *use)
+static int use_pcg(sim_handle *h, bool *use, cudaStream_t s)
 {
     *use = false;
     if (h->opt.cg_kernel != SIM_CG_AUTO || h->timing) return SIM_OK;
     if (h->pcg_state == 0) {
         int rc = SIM_OK;
         try {
-            rc = build_pcg<T>(h);
+            rc = build_pcg<T>(h, s);
         } catch (const std::exception &) {  // no host memory for the plan: per-iteration kernels
             h->pcg_state = -1;
         }
@@ -858,7 +861,7 @@ static int newton_impl(sim_handle *h, bool dyn, sim_solve_stats *st, cudaStream_
         return S.status;
     }
     bool pcg;
-    if ((rc = use_pcg<T>(h, &pcg))) return rc;
+    if ((rc = use_pcg<T>(h, &pcg, s))) return rc;
     if (!pcg) launch_record_activation<T>(c, s);
     const double eps = 2.220446049250313e-16;
     int it = 0;
@@ -995,7 +998,7 @@ static int adjoint_impl(sim_handle *h, bool dyn, const double *b, double *lambda
         return S.status;
     }
     bool pcg;
-    if ((rc = use_pcg<T>(h, &pcg))) return rc;
+    if ((rc = use_pcg<T>(h, &pcg, s))) return rc;
     if (!pcg) launch_record_activation<T>(c, s);
     double rn = bn;
     const double target = h->opt.adjoint_rtol * bn;
