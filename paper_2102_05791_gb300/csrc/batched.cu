@@ -227,7 +227,7 @@ static int build_plans(sim_batch *bt, const sim_mesh *meshes, const std::vector<
         if (a > c) a = c * aggregates_per_part((nv[m] + c - 1) / c, a / c, bt->threads);
         ok[m] = build_cg_plan(d, nv[m], ne[m], meshes[m].rest_pos, meshes[m].elems, perm.data(), ne[m], c, a, true,
                               sizeof(float), false, plans[m], err) &&
-                plans[m].ns <= kBatchVpt * bt->threads && plans[m].max_items <= 16;
+                batch_plan_fits(plans[m], bt->threads);
         if (!ok[m]) return;
         pcg_sizes_of(plans[m], c > 1, true, pds[m]);
         pds[m].threads = bt->threads;

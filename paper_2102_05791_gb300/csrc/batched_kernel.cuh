@@ -72,9 +72,6 @@ struct Mesh {
     bool planned;         // its CG solves have a plan (else they run matrix-free)
 };
 
-constexpr int kBatchPlanAt = kPcgSmem - kPcgStatic;  // dynamic shared memory of the plan's layout
-constexpr int kBatchVpt = 8;                         // vertices of a mesh per thread at most
-
 namespace {
 
 // Dynamic shared memory: the plan's layout (PcgSmem), then the mesh's PcgDev.
@@ -592,7 +589,7 @@ __device__ __noinline__ void assemble(const BatchDev &b, const Mesh &m, Team &tm
         }
         tm.sync();
         if (tm.rank == 0) {
-            // Gauss-Jordan in shared memory, scaled to unit diagonal (as k_coarse_invert)
+            // Gauss-Jordan in shared memory (batch_plan_fits has its size), scaled to unit diagonal (as k_coarse_invert)
             float *A = reinterpret_cast<float *>(batch_smem + L.ring), *scale = A + N * N, *row = scale + N, *col = row + N;
             for (int k = threadIdx.x; k < N; k += blockDim.x) {
                 const float d = pd.E[(size_t)k * N + k];

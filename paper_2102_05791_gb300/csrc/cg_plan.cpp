@@ -121,6 +121,15 @@ int aggregates_per_part(int64_t v, int most, int threads)
     return best;
 }
 
+bool batch_plan_fits(const CgPlan &P, int threads)
+{
+    const size_t N = (size_t)P.n_agg * P.n_modes, esz = 4 + (size_t)P.dim * P.dim * sizeof(float);
+    const PcgSmem L(P.dim, sizeof(float), P.ns, P.max_halo, P.max_items, (int)N, P.n_meta, 0);
+    return P.ns <= kBatchVpt * threads && P.max_items <= 16 && N <= (size_t)kCgMaxCoarse &&
+           L.ring + sizeof(float) * (N * N + 3 * N) <= (size_t)kBatchPlanAt &&
+           L.ring + (size_t)P.max_entries * esz <= (size_t)kBatchPlanAt;
+}
+
 bool build_cg_plan(int dim, int64_t nv, int64_t ne, const double *X, const int32_t *T, const int32_t *perm,
                    int64_t ne_int, int n_cta, int n_agg, bool rows, int elt, bool on_grid, CgPlan &P, std::string &err)
 {

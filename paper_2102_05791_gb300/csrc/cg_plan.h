@@ -112,6 +112,16 @@ struct CgPlan {
 // slots, else the least wasteful.
 int aggregates_per_part(int64_t v, int most, int threads);
 
+// The batched solver: dynamic shared memory of the plan's layout (the body's
+// plan record lies behind it), and vertices of a body per thread at most.
+constexpr int kBatchPlanAt = kPcgSmem - kPcgStatic;
+constexpr int kBatchVpt = 8;
+
+// Whether a body's plan (FP32, by rows) fits the batched kernel with that many
+// threads: its slots, its aggregates, and below the plan record the edge slice
+// and, in the same place, the scratch the coarse matrix is inverted in.
+bool batch_plan_fits(const CgPlan &P, int threads);
+
 // rows: store the parts by rows; elt: bytes of a value of the solver; on_grid: the
 // CTAs are not one cluster.  perm: tile order -> caller order (-1 padding), ne_int entries; max_entries of any CTA
 // and halo sizes are left to the caller to check against shared memory.  Returns false
