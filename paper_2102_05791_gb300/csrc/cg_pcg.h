@@ -48,8 +48,8 @@ template <typename T>
 void launch_pcg_assemble(const Ctx &c, const PcgDev &pd, const Phys &ph, const T *u, const double *u64, bool coarse,
                          cudaStream_t s);
 
-// Shared memory of the solver and whether the slice is streamed: fills threads, vpt, stages and
-// cluster; false when a CTA's vectors do not fit.
+// Shared memory of the solver and whether the slice is streamed: fills threads, vpt and stages;
+// false when a CTA's vectors do not fit, or the device cannot hold all CTAs at once.
 template <typename T>
 bool pcg_configure(const Ctx &c, PcgDev &pd);
 

@@ -158,6 +158,50 @@ static void *pcg_kernel(int vpt, bool rows)
     }
 }
 
+// The launch of a configured plan, in place; at[1] is filled in too.
+template <typename T>
+static cudaLaunchConfig_t pcg_launch_config(int dim, const PcgDev &pd, cudaLaunchAttribute *at, cudaStream_t s)
+{
+    const size_t esz = 4 + dim * dim * sizeof(T);
+    const bool on_grid = pd.n_cta > 1 && !pd.cluster;
+    const PcgSmem L(dim, sizeof(T), pd.ns, pd.max_halo, pd.max_items, pd.n_coarse, pd.n_meta, on_grid ? pd.n_cta : 0);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(pd.n_cta);
+    cfg.blockDim = dim3(pd.threads + (pd.stages ? 32 : 0));
+    cfg.dynamicSmemBytes = L.ring + (pd.stages ? (size_t)pd.stages * kCgChunk * esz : (size_t)pd.max_entries * esz);
+    cfg.stream = s;
+    cfg.attrs = at;
+    if (pd.cluster) {  // one cluster: every CTA co-scheduled by construction
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = pd.n_cta;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.numAttrs = 1;
+    } else if (on_grid) {
+        at[0].id = cudaLaunchAttributeCooperative;
+        at[0].val.cooperative = 1;
+        cfg.numAttrs = 1;
+    }
+    return cfg;
+}
+
+// Whether the device can hold all CTAs of the configured launch at once.
+template <typename T>
+static bool resident(int dim, const PcgDev &pd, const void *k)
+{
+    cudaLaunchAttribute at[1];
+    const cudaLaunchConfig_t cfg = pcg_launch_config<T>(dim, pd, at, nullptr);
+    int clusters = 0, per_sm = 0, dev = 0, sms = 0;
+    cudaError_t e;
+    if (pd.cluster) {
+        e = cudaOccupancyMaxActiveClusters(&clusters, k, &cfg);
+    } else {
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, (int)cfg.blockDim.x, cfg.dynamicSmemBytes);
+        if (e == cudaSuccess) e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    }
+    return e == cudaSuccess && pcg_resident(pd.cluster != 0, pd.n_cta, clusters, per_sm, sms);
+}
+
 template <typename T, int D>
 static bool configure(const Ctx &c, PcgDev &pd)
 {
@@ -184,14 +228,17 @@ static bool configure(const Ctx &c, PcgDev &pd)
             break;
         if (!streamed) {
             pd.stages = 0;
-            if (base.ring + (size_t)pd.max_entries * esz <= limit) return true;
-            if (pd.cluster) return false;
+            if (base.ring + (size_t)pd.max_entries * esz > limit) {
+                if (pd.cluster) return false;
+                continue;
+            }
         } else {
             if (base.ring + 3 * kCgChunk * esz > limit) return false;
             pd.stages = (int)((limit - base.ring) / (kCgChunk * esz));
             if (pd.stages > kPcgMaxStages) pd.stages = kPcgMaxStages;
-            return true;
         }
+        if (resident<T>(D, pd, k)) return true;
+        break;
     }
     cudaGetLastError();
     return false;
@@ -207,34 +254,15 @@ template <typename T>
 cudaError_t launch_pcg(const Ctx &c, const PcgDev &pd, const double *b, double sign, T *d, double rtol, int max_iter,
                        cudaStream_t s)
 {
-    const size_t esz = 4 + c.dim * c.dim * sizeof(T);
-    const size_t slice = pd.stages ? (size_t)pd.stages * kCgChunk * esz : (size_t)pd.max_entries * esz;
-    const bool on_grid = pd.n_cta > 1 && !pd.cluster;
-    const size_t sm = PcgSmem(c.dim, sizeof(T), pd.ns, pd.max_halo, pd.max_items, pd.n_coarse, pd.n_meta,
-                              on_grid ? pd.n_cta : 0).ring + slice;
     void *k = c.dim == 2 ? pcg_kernel<T, 2>(pd.vpt, pd.tpr > 0) : pcg_kernel<T, 3>(pd.vpt, pd.tpr > 0);
     int polls = c.td.wait_polls;
     DevScalars *sc = c.sc;
     void *args[] = {(void *)&pd, (void *)&b, &sign, &d, &rtol, &max_iter, &polls, &sc};
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(pd.n_cta);
-    cfg.blockDim = dim3(pd.threads + (pd.stages ? 32 : 0));
-    cfg.dynamicSmemBytes = sm;
-    cfg.stream = s;
     cudaLaunchAttribute at[1];
-    cfg.attrs = at;
-    cfg.numAttrs = 0;
-    if (pd.cluster) {  // one cluster: every CTA co-scheduled by construction
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = pd.n_cta;
-        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-        cfg.numAttrs = 1;
-    } else if (pd.n_cta > 1) {
+    const cudaLaunchConfig_t cfg = pcg_launch_config<T>(c.dim, pd, at, s);
+    if (pd.n_cta > 1 && !pd.cluster) {
         const cudaError_t e = cudaMemsetAsync(pd.words, 0, (size_t)16 * kPcgWords * pd.n_cta, s);
         if (e != cudaSuccess) return e;
-        at[0].id = cudaLaunchAttributeCooperative;
-        at[0].val.cooperative = 1;
-        cfg.numAttrs = 1;
     }
     c.n_launch += 1;
     return cudaLaunchKernelExC(&cfg, k, args);

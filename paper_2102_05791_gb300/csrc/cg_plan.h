@@ -76,6 +76,14 @@ struct PcgSmem {
     }
 };
 
+// Whether a launch of n_cta CTAs that wait for one another may be made: one
+// cluster when the device can hold at least one of its kind, else a grid of at
+// most the CTAs that fit on its SMs together.
+inline bool pcg_resident(bool cluster, int n_cta, int max_clusters, int per_sm, int sms)
+{
+    return cluster ? max_clusters >= 1 : n_cta <= (int64_t)per_sm * sms;
+}
+
 struct CgPlan {
     int dim = 0, n_cta = 0, n_agg = 0, n_modes = 0;
     int ns = 0;                        // slots per CTA (maximum over CTAs, a multiple of 32)

@@ -737,7 +737,7 @@ static int build_pcg(sim_handle *h, cudaStream_t s)
     PcgDev &pd = h->pcg;
     pcg_sizes_of(P, z.cluster, h->mat.dt > 0.0 || h->mat.k_contact > 0.0, pd);
     if (!pcg_configure<T>(h->ctx, pd)) {
-        if (h->verbose) fprintf(stderr, "[softsim] per-iteration CG kernels: a part does not fit in shared memory\n");
+        if (h->verbose) fprintf(stderr, "[softsim] per-iteration CG kernels: the parts do not fit on the device\n");
         return SIM_OK;
     }
     // one allocation for the plan's tables and one for the buffers: forty separate ones cost milliseconds
