@@ -14,7 +14,8 @@
 // team takes it.
 //
 // Precision follows the single-mesh mixed path: FP32 HVP and CG vectors,
-// FP64 state, gradient, energies, dot products and adjoint residuals.
+// FP64 state, gradient, energies and adjoint residuals, compensated FP32 dot
+// products in CG.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>

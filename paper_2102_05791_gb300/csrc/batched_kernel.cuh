@@ -353,7 +353,7 @@ __device__ __noinline__ double energy_pass(const BatchDev &b, const Mesh &m, Tea
 }
 
 // y = (M + h^2 H(u)) v with pinned rows/columns dropped; returns v.y (FP64
-// sum for T = double, compensated FP32 block sum for T = float).
+// sum, of FP32 terms per thread for T = float).
 template <typename T, int D>
 __device__ __noinline__ double hvp_pass(const BatchDev &b, const Mesh &m, Team &tm, const double *a_t, const T *us, const T *v, T *y, T *c,
                            const T *ed)
@@ -647,8 +647,8 @@ __device__ __noinline__ int cg_assembled(const double *rhs, double rhs2, float *
     __shared__ int never_bad;  // the slice is in place: no copy to wait for
     if (threadIdx.x == 0) never_bad = 0;
     Slice sl = pcg_slice<D, float, true>(plan(), rank, false, batch_smem, 0, &never_bad);
-    return pcg_run<float, D, VPT, true>(plan(), sl, rank, false, batch_smem, rhs, 1.0, rhs2, d, rtol, max_it,
-                                        new_coarse).iter;
+    return pcg_run<float, D, VPT, true, false>(plan(), sl, rank, batch_smem, rhs, 1.0, rhs2, d, rtol, max_it,
+                                               new_coarse).iter;
 }
 
 // CG on (M + h^2 H) d = rhs (|rhs|^2 = rhs2) with the assembled operator, or

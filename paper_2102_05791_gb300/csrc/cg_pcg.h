@@ -36,7 +36,7 @@ struct PcgDev {
     float4 *pos4 = nullptr;          // [n_cta*ns] rotation arm of a slot (scaled), aggregate | pinned << 30
     void *diag2 = nullptr;           // [n_cta*ns][2] vertex diagonal: horizontal axes, y
     void *dinv = nullptr;            // [6 or 3][n_cta*ns] inverse diagonal blocks
-    void *zr = nullptr;              // [n_cta*ns][4 or 2] published D^-1 r
+    void *zr = nullptr;              // [n_cta*ns][4 or 2] published z
     float *cpart = nullptr;          // [n_citems][36]
     float *E = nullptr, *Einv = nullptr;  // [n_coarse][n_coarse]
     unsigned long long *words = nullptr;          // [2][n_cta][kPcgWords] (value, tag) words of a grid's exchanges

@@ -4,6 +4,7 @@
 #pragma once
 
 #include <cstdint>
+#include <type_traits>
 
 #include "cg_pcg.h"
 #include "grid_sync.cuh"
@@ -167,6 +168,104 @@ __device__ __forceinline__ void sym_mul(const T *S, const T r[D], T z[D])
     }
 }
 
+// Inner products of the solver.  FP32: a pair (hi, lo) whose sums are all
+// compensated (TwoSum, Knuth), about 48 bits where FP64 would cost 64 times the
+// issue slots; FP64: a double.
+template <typename T>
+struct DotOf {
+    using Type = double;
+};
+template <>
+struct DotOf<float> {
+    using Type = float2;
+};
+
+// s + e == a + b exactly, in intrinsics: contracting a product into the sum would lose its error.
+__device__ __forceinline__ void two_sum_rn(float a, float b, float &s, float &e)
+{
+    s = __fadd_rn(a, b);
+    const float bb = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+
+// v += x . y of one vertex.  EXACT: with the rounding errors of the products
+// too (dot product of Ogita, Rump and Oishi 2005), else they come from one FMA
+// chain.  first: v is zero.
+template <int D, bool EXACT>
+__device__ __forceinline__ void dot_add(float2 &v, const float *x, const float *y, bool first)
+{
+    float p = __fmul_rn(x[0], y[0]), e = 0.0f;
+    if (EXACT) e = __fmaf_rn(x[0], y[0], -p);
+#pragma unroll
+    for (int c = 1; c < D; ++c) {
+        if (EXACT) {
+            const float q = __fmul_rn(x[c], y[c]), eq = __fmaf_rn(x[c], y[c], -q);
+            float es;
+            two_sum_rn(p, q, p, es);
+            e = __fadd_rn(e, __fadd_rn(eq, es));
+        } else {
+            p = __fmaf_rn(x[c], y[c], p);
+        }
+    }
+    if (first) {
+        v = make_float2(p, e);
+        return;
+    }
+    float es;
+    two_sum_rn(v.x, p, v.x, es);
+    v.y = __fadd_rn(v.y, __fadd_rn(e, es));
+}
+template <int D, bool EXACT>
+__device__ __forceinline__ void dot_add(double &v, const double *x, const double *y, bool)
+{
+#pragma unroll
+    for (int c = 0; c < D; ++c) v += x[c] * y[c];
+}
+
+// The sum of two partial dots; the same bits whichever comes first.
+__device__ __forceinline__ float2 dot_merge(float2 a, float2 b)
+{
+    float2 r;
+    two_sum(a.x, b.x, r.x, r.y);
+    r.y += a.y + b.y;
+    return r;
+}
+
+__device__ __forceinline__ double dot_merge(double a, double b) { return a + b; }
+
+__device__ __forceinline__ float2 dot_xor(float2 v, int o)
+{
+    return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
+}
+__device__ __forceinline__ double dot_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+
+// Sums over groups of 2 K lanes, the same in every lane of a group.  (Two digits of
+// fixed point added by the integer reduction instructions instead of the shuffles:
+// slower, 4.3 to 4.6 us an iteration on the walker.)
+template <int K, typename V>
+__device__ __forceinline__ V group_dot(V v)
+{
+#pragma unroll
+    for (int o = K; o > 0; o >>= 1) v = dot_merge(v, dot_xor(v, o));
+    return v;
+}
+
+// The dot rounded to FP32.
+__device__ __forceinline__ float dot_value(float2 v) { return v.x + v.y; }
+__device__ __forceinline__ double dot_value(double v) { return v; }
+
+// a / b rounded to FP32: a quotient good to a few units and the remainder it leaves.
+__device__ __forceinline__ float dot_quot(float2 a, float2 b)
+{
+    const float bv = dot_value(b), q = __fdividef(dot_value(a), bv);
+    const float r = __fadd_rn(__fmaf_rn(-q, b.x, a.x), __fmaf_rn(-q, b.y, a.y));
+    return __fadd_rn(q, __fdividef(r, bv));
+}
+
+// a - b rounded to FP32 (exact in sign for dots that agree in their leading parts).
+__device__ __forceinline__ float dot_minus(float2 a, float2 b) { return (a.x - b.x) + (a.y - b.y); }
+__device__ __forceinline__ double dot_minus(double a, double b) { return a - b; }
+
 // What a CTA's threads share in the edge passes.
 struct Slice {
     unsigned char *base;             // the slice in shared memory, or the ring
@@ -290,7 +389,9 @@ template <typename V>
 __device__ __forceinline__ void st_dsmem(void *local, uint32_t rank, V v)
 {
     const uint32_t a = dsmem_addr(local, rank);
-    if constexpr (sizeof(V) == 4)
+    if constexpr (std::is_same_v<V, float2>)
+        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+    else if constexpr (sizeof(V) == 4)
         asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
     else
         asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
@@ -387,30 +488,31 @@ struct PcgResult {
 // The solve itself, by the consumer threads of one CTA (number cta of pd.n_cta)
 // whose slice sl and tables (pcg_tables) are in place: x with A x = sign b to
 // |r| <= rtol |b| goes to dout.  ROWS: the slice is stored by rows (see
-// cg_plan.h), else by colours.  grid: the CTAs are a grid, else one cluster or
-// one CTA; nb2: |b|^2;
-// new_coarse: the coarse
-// inverse is not the one of the CTA's previous solve.
-template <typename T, int D, int VPT, bool ROWS>
-__device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int cta, bool grid, unsigned char *smem,
-                                             const double *b, double sign, double nb2, T *dout, double rtol,
-                                             int max_iter, bool new_coarse)
+// cg_plan.h), else by colours.  GRID: the CTAs are a grid, else one cluster or
+// one CTA (a variant of its own: the grid's exchange would cost a cluster's
+// solver its registers, 4.2 to 4.4 us an iteration on the walker); nb2: |b|^2;
+// new_coarse: the coarse inverse is not the one of the CTA's previous solve.
+template <typename T, int D, int VPT, bool ROWS, bool GRID>
+__device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int cta, unsigned char *smem, const double *b,
+                                             double sign, double nb2, T *dout, double rtol, int max_iter,
+                                             bool new_coarse)
 {
+    constexpr bool grid = GRID;
     constexpr int NM = D == 3 ? 6 : 3, ND = D == 3 ? 6 : 3, DD = D * D, RN = Row<T, D>::N;
     constexpr int NI = (NM + 1) / 2;       // pairs of words that hold a CTA's items
     constexpr bool F32 = sizeof(T) == 4;
+    using Dot = typename DotOf<T>::Type;
     // A slot's arm, vertex diagonal and inverse block stay in registers where one
     // slot a thread leaves room (walker 4.54 -> 4.09 us an iteration, 70,785
     // vertices 13.0 -> 12.5); with four slots the spills cost more than the loads
     // (2D 20,000 vertices 7.1 -> 7.6 us)
     constexpr bool KEEP_S = F32 && VPT == 1;
-    constexpr bool KEEP_Z = VPT <= 2;  // so does D^-1 r between the phases
-    constexpr int VB = VPT < 2 ? VPT : 2;  // slots whose loads are issued together
-    constexpr int PB = VPT < 4 ? 4 : 2;    // loads of an exchange in flight per thread
-    __shared__ float sred[kMaxWarps * VPT][8];  // per warp, or per group of 32 slots: restriction, two dots
+    constexpr bool EXACT = VPT <= 2;   // with more slots the products' errors average out (largest body: 61.6 us with, 60.2 without)
+    constexpr bool KEEP_Z = VPT <= 2;  // so does z between the phases
+    __shared__ float sred[kMaxWarps * VPT][8];  // restriction, per warp or per group of 32 slots
     __shared__ T sbc[3];
-    __shared__ T sdot[2][kMaxWarps];            // the dots of the FP64 solver
-    __shared__ T sdots[3][kMaxWarps];           // dots of the CTAs of a cluster (or of the only CTA)
+    __shared__ Dot sdot[2][kMaxWarps];          // dots of the warps
+    __shared__ Dot sdots[3][kMaxWarps];         // dots of the CTAs of a cluster (or of the only CTA), or of 32 CTAs of a grid
     __shared__ float scown[kMaxWarps][8];       // coarse values of this CTA's aggregates
     __shared__ int sgrp[kMaxWarps + 1];         // first group of 32 slots of an item
     __shared__ int sok;
@@ -420,13 +522,15 @@ __device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int ct
     const int nh = pd.halo_ptr[cta + 1] - pd.halo_ptr[cta];
     const int i0 = pd.item_ptr[cta], ni = pd.item_ptr[cta + 1] - i0, a0 = pd.item_agg[i0];
     const bool one = ni == 1, solo = G == 1;
+    constexpr int PB = VPT < 4 ? 4 : 2;    // loads of an exchange in flight per thread
+    const int n_part = grid ? (G + 31) / 32 : 1;  // partial sums of a dot over a grid's CTAs
     const PcgSmem L(D, sizeof(T), pd.ns, pd.max_halo, pd.max_items, N, pd.n_meta, grid ? G : 0);
     T *sp = reinterpret_cast<T *>(smem + L.p), *sy = reinterpret_cast<T *>(smem + L.y);
-    float *sE = reinterpret_cast<float *>(smem + L.e), *sc_ = reinterpret_cast<float *>(smem + L.c);
+    float *sE = reinterpret_cast<float *>(smem + L.e);
     // ss: restricted residual, two buffers (a cluster's CTAs write the next one while this one is read)
     float *ss = reinterpret_cast<float *>(smem + L.s), *ss_next = ss + N, *st_ = reinterpret_cast<float *>(smem + L.t);
     const int32_t *shalo = reinterpret_cast<const int32_t *>(smem + L.halo);
-    uint32_t *sword = reinterpret_cast<uint32_t *>(smem + L.word);  // [G][kPcgWords] of a grid's exchange
+    uint32_t *sword = reinterpret_cast<uint32_t *>(smem + L.word);  // [G][kPcgRow] of a grid's exchange
     int fail = 0;
     for (int k = tid; k < kMaxWarps * VPT * 8; k += nthr) (&sred[0][0])[k] = 0.0f;
     for (int k = tid; k < ns / 32; k += nthr) {
@@ -506,39 +610,50 @@ __device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int ct
         const int g = k < ns ? gid(k) : -1;
         return g >= 0 && !(__float_as_int(pos(k).w) >> 30) ? sign * b[(int64_t)g * D + c] : 0.0;
     };
-    // Per-slot reduction values v: NM restricted components, then up to two
-    // dots (FP32 solver).  A CTA of one aggregate sums its slots first.
+    // Per-slot restricted components v (v[6], v[7] are zero).  A CTA of one
+    // aggregate sums its slots first.
     auto put_sum = [&](int m, const float v[8]) {
         const float t = warp_sum8(v);
         if ((lane & 3) == 0) sred[one ? wrp : m * nw + wrp][lane >> 2] = t;
     };
-    // The CTA's nd dots (after put_sum): valid in the lanes < nd of the last warp.
-    auto cta_dot = [&](int nd) -> T {
-        T v = T(0);
-        if constexpr (F32) {
-            const int q = 6 + (lane & 1), h = lane >> 1, ng = one ? nw : ns / 32;
-            for (int g = h; g < ng; g += 16) v += sred[g][q];
+    auto put_group = [&](int m, float v[8]) {  // of one group of 32 slots
+        put_sum(m, v);
 #pragma unroll
-            for (int o = 16; o > 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        } else if (lane < nd) {
-            for (int w = 0; w < nw; ++w) v += sdot[lane][w];
+        for (int q = 0; q < 8; ++q) v[q] = 0.0f;
+    };
+    // Two dots share a warp's sum: the lower half-warp ends with the first, the
+    // upper with the second (of one dot, both with it).
+    auto half = [&](int nd) { return nd > 1 ? lane >> 4 : 0; };
+    auto dot_of = [&](Dot v, int d) -> Dot {
+        if constexpr (F32)
+            return make_float2(__shfl_sync(0xffffffffu, v.x, 16 * d), __shfl_sync(0xffffffffu, v.y, 16 * d));
+        else
+            return __shfl_sync(0xffffffffu, v, 16 * d);
+    };
+    // This warp's nd dots to shared memory; warps without slots have none.
+    auto put_dots = [&](int nd, const Dot *dots) {
+        Dot v{};
+        if (wrp * 32 < ns && nd > 0) {
+            const bool up = half(nd) != 0, low = nd > 1 && !up;
+            v = dot_merge(up ? dots[1] : dots[0], dot_xor(low ? dots[1] : dots[0], 16));
+            v = group_dot<8>(v);
         }
-        return v;
+        if ((lane & 15) == 0 && (lane >> 4) < nd) sdot[lane >> 4][wrp] = v;
+    };
+    // The CTA's nd dots (after put_dots), by one warp.
+    auto cta_dot = [&](int nd) -> Dot {
+        const int w = lane & 15;
+        return group_dot<8>(w < nw ? sdot[half(nd)][w] : Dot{});
     };
     // Exchange of the restricted vector (into dst) and of nd dots (slot base of
-    // sdots, or words of the grid); also of the coarse values with with_c.  buf
-    // and tag name the grid's words; fence orders the rows published before.
-    auto exchange = [&](int nd, const T *dots, float *dst, bool with_c, int base, int buf, uint32_t tag) -> bool {
-        if constexpr (!F32) {
-            for (int q = 0; q < nd; ++q) {
-                const T v = wrp * 32 < ns ? warp_all(dots[q]) : T(0);  // the FP64 pipe is the bottleneck: no sums of zeros
-                if (lane == 0) sdot[q][wrp] = v;
-            }
-        }
+    // sdots, or words of the grid).  rows: the CTA has published its rows of z,
+    // which others read after it.  buf and tag name the grid's words.
+    auto exchange = [&](int nd, const Dot *dots, float *dst, bool rows, int base, int buf, uint32_t tag) -> bool {
+        put_dots(nd, dots);
         csync(nthr);
         const int q = lane & 7, h = lane >> 3;
         unsigned long long *mine = pd.words + ((size_t)buf * G + cta) * kPcgWords;
-        if (grid && with_c && wrp == 0) __threadfence();  // the CTA's rows before its words
+        if (grid && rows && wrp == 0) __threadfence();  // the CTA's rows before its words
         for (int it = wrp; it < ni; it += nw) {
             float v = 0.0f;
             if (one) {
@@ -551,38 +666,33 @@ __device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int ct
             v += __shfl_xor_sync(0xffffffffu, v, 16);
             if (grid) {  // one aggregate a CTA
                 if (h == 0 && q < 2 * NI) put_word(mine + q, __float_as_uint(v), tag);
-                if (with_c && h == 1 && q < 2 * NI) put_word(mine + 8 + q, q < NM ? __float_as_uint(scown[0][q]) : 0u, tag);
             } else if (q < NM) {
                 const int n = (a0 + it) * NM + q;
-                const float c = with_c ? scown[it][q] : 0.0f;
                 if (solo) {
-                    dst[n] = v;
-                    if (with_c) sc_[n] = c;
+                    if (h == 0) dst[n] = v;
                 } else {
-                    for (int k = h; k < G; k += 4) {
-                        st_dsmem(dst + n, (uint32_t)k, v);
-                        if (with_c) st_dsmem(sc_ + n, (uint32_t)k, c);
-                    }
+                    for (int k = h; k < G; k += 4) st_dsmem(dst + n, (uint32_t)k, v);
                 }
             }
         }
         if (nd > 0 && wrp == nw - 1) {
-            const T v = cta_dot(nd);
-            if (grid) {
-                if (lane < (F32 ? 2 : nd)) {
-                    if constexpr (F32) {
-                        put_word(mine + 14 + lane, __float_as_uint(v), tag);
-                    } else {
-                        put_word(mine + 14 + 2 * lane, (uint32_t)__double2loint(v), tag);
-                        put_word(mine + 15 + 2 * lane, (uint32_t)__double2hiint(v), tag);
-                    }
+            const Dot v = cta_dot(nd);
+            if (!grid && !solo) {
+                for (int k = 0; k < nd; ++k) {
+                    const Dot w = dot_of(v, k);
+                    if (lane < G) st_dsmem(&sdots[base + k][cta], (uint32_t)lane, w);
                 }
-            } else if (solo) {
-                if (lane < nd) sdots[base + lane][0] = v;
             } else {
-                for (int d = 0; d < nd; ++d) {
-                    const T w = __shfl_sync(0xffffffffu, v, d);
-                    if (lane < G) st_dsmem(&sdots[base + d][cta], (uint32_t)lane, w);
+                const int d = lane >> 4, i = lane & 15;
+                if (solo) {
+                    if (d < nd && i == 0) sdots[base + d][0] = v;
+                } else {  // two words a dot, from neighbouring lanes: the parts of a pair, or the halves of a double
+                    uint32_t w;
+                    if constexpr (F32)
+                        w = __float_as_uint(i ? v.y : v.x);
+                    else
+                        w = (uint32_t)(i ? __double2hiint(v) : __double2loint(v));
+                    if (d < nd && i < 2) put_word(mine + kPcgDots + 2 * d + i, w, tag);
                 }
             }
         }
@@ -594,95 +704,89 @@ __device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int ct
             cluster_sync();
             return true;
         }
-        // the words of every CTA (items and dots) and, with_c, the coarse values of
-        // every aggregate's first CTA; PB loads in flight before the first is looked at
+        // the words of every CTA, neighbouring threads on one CTA's line; PB loads in
+        // flight before the first is looked at
         const unsigned long long *all = pd.words + (size_t)buf * G * kPcgWords;
-        const int nt = NI + (F32 ? (nd > 0) : nd), n_cta_load = G * nt, n_load = n_cta_load + (with_c ? pd.n_agg * NI : 0);
-        auto at = [&](int k) {
-            if (k >= n_cta_load) {
-                const int a = (k - n_cta_load) / NI;
-                return pd.agg_item[a] * kPcgWords + 8 + 2 * (k - n_cta_load - a * NI);
-            }
-            const int g = k / nt, j = k - g * nt;
-            return g * kPcgWords + 2 * (j < NI ? j : 7 + j - NI);
-        };
+        const int nt = NI + nd, n_load = G * nt;
         bool ok = true;
         for (int k0 = tid; k0 < n_load; k0 += PB * nthr) {
             ulonglong2 w[PB];
-            int o[PB];
+            int o[PB];  // CTA << 8 | word
 #pragma unroll
             for (int u = 0; u < PB; ++u)
                 if (k0 + u * nthr < n_load) {
-                    o[u] = at(k0 + u * nthr);
-                    w[u] = load_words(all + o[u]);
+                    const int k = k0 + u * nthr, g = k / nt, j = k - g * nt;
+                    o[u] = g << 8 | (j < NI ? 2 * j : kPcgDots + 2 * (j - NI));
+                    w[u] = load_words(all + g * kPcgWords + (o[u] & 255));
                 }
 #pragma unroll
             for (int u = 0; u < PB; ++u) {
                 if (k0 + u * nthr >= n_load) break;
                 for (int i = 0; ok && ((uint32_t)(w[u].x >> 32) != tag || (uint32_t)(w[u].y >> 32) != tag); ++i) {
                     if (i >= kGridWaitPolls) ok = false;
-                    w[u] = load_words(all + o[u]);
+                    w[u] = load_words(all + (o[u] >> 8) * kPcgWords + (o[u] & 255));
                 }
-                sword[o[u]] = (uint32_t)w[u].x;
-                sword[o[u] + 1] = (uint32_t)w[u].y;
+                *reinterpret_cast<uint2 *>(sword + (o[u] >> 8) * kPcgRow + (o[u] & 255)) =
+                    make_uint2((uint32_t)w[u].x, (uint32_t)w[u].y);
             }
         }
         if (!ok) sok = 0;
-        if (with_c) __threadfence();  // the rows read next are those published before the words
+        if (rows) __threadfence();  // the rows read next are those published before the words
         csync(nthr);
         for (int n = tid; n < N; n += nthr) {
             const int a = n / NM, j = n - a * NM, g0 = pd.agg_item[a], g1 = pd.agg_item[a + 1];
             float v = 0.0f;
-            for (int g = g0; g < g1; ++g) v += __uint_as_float(sword[g * kPcgWords + j]);
+            for (int g = g0; g < g1; ++g) v += __uint_as_float(sword[g * kPcgRow + j]);
             dst[n] = v;
-            if (with_c) sc_[n] = __uint_as_float(sword[g0 * kPcgWords + 8 + j]);
+        }
+        for (int u = nw - 1 - wrp; u < nd * n_part; u += nw) {  // meanwhile the last warps: a dot over 32 CTAs each
+            const int d = u >= n_part, p = u - d * n_part, g = p * 32 + lane;
+            Dot v{};
+            if (g < G) {
+                const uint2 w = *reinterpret_cast<const uint2 *>(sword + g * kPcgRow + kPcgDots + 2 * d);
+                if constexpr (F32)
+                    v = make_float2(__uint_as_float(w.x), __uint_as_float(w.y));
+                else
+                    v = __hiloint2double((int)w.y, (int)w.x);
+            }
+            v = group_dot<16>(v);
+            if (lane == 0) sdots[base + d][p] = v;
         }
         csync(nthr);
         return sok != 0;
     };
-    // This lane's share of dot d of the last exchange (every warp sums the CTAs alike).
-    auto dot_part = [&](int base, int d) -> T {
-        T v = T(0);
-        if (!grid) {
-            if (lane < G) v = sdots[base + d][lane];
+    // Sums of the nd dots of the last exchange over the CTAs; every calling warp forms them alike.
+    auto dot_sums = [&](int base, int nd, Dot *out) {
+        if (grid || solo) {
+            for (int d = 0; d < nd; ++d) out[d] = sdots[base + d][0];
+            for (int p = 1; p < n_part; ++p)
+                for (int d = 0; d < nd; ++d) out[d] = dot_merge(out[d], sdots[base + d][p]);
         } else {
-            for (int g = lane; g < G; g += 32) {
-                if constexpr (F32)
-                    v += __uint_as_float(sword[g * kPcgWords + 14 + d]);
-                else
-                    v += __hiloint2double((int)sword[g * kPcgWords + 15 + 2 * d], (int)sword[g * kPcgWords + 14 + 2 * d]);
-            }
+            const int g = lane & 15;
+            const Dot v = group_dot<8>(g < G ? sdots[base + half(nd)][g] : Dot{});
+            for (int d = 0; d < nd; ++d) out[d] = dot_of(v, d);
         }
-        return v;
     };
     auto swap_s = [&]() {
         float *t = ss;
         ss = ss_next;
         ss_next = t;
     };
-    auto coarse_part = [&]() -> T {  // Z^T r . c
-        float v = 0.0f;
-#pragma unroll
-        for (int u = 0; u < kCgMaxCoarse / 32; ++u) {
-            const int n = lane + 32 * u;
-            if (n < N) v = fmaf(ss[n], sc_[n], v);
-        }
-        return T(v);
-    };
     // The coarse values of this CTA's aggregates from the restricted residual ss
-    // - alpha st_: a warp per row of E^-1, or, with more rows than warps, eight
-    // lanes per row.
+    // - alpha st_: a warp per row of E^-1 (the last ones, which often have no
+    // slots), or, with more rows than warps, eight lanes per row.
     auto coarse = [&](float alpha, bool with_t) {
         if (ni * NM <= nw) {
-            if (wrp < ni * NM) {
+            const int row = nw - 1 - wrp;
+            if (row < ni * NM) {
                 float v = 0.0f;
 #pragma unroll
                 for (int u = 0; u < kCgMaxCoarse / 32; ++u) {
                     const int n = lane + 32 * u;
-                    if (n < N) v = fmaf(sE[wrp * N + n], with_t ? fmaf(-alpha, st_[n], ss[n]) : ss[n], v);
+                    if (n < N) v = fmaf(sE[row * N + n], with_t ? fmaf(-alpha, st_[n], ss[n]) : ss[n], v);
                 }
                 v = warp_all(v);
-                if (lane == 0) scown[wrp / NM][wrp % NM] = v;
+                if (lane == 0) scown[row / NM][row % NM] = v;
             }
         } else {
             const int sub = lane & 7;
@@ -737,57 +841,71 @@ __device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int ct
 #pragma unroll
         for (int c = 0; c < D; ++c) x[m][c] = T(0);
     int it = 0, neg = 0;
-    T rr = T(1), rz = T(0);
-    const T tol2 = T(rtol * rtol);
+    Dot rr{}, rz{};
+    // rtol^2 |b|^2 with |b| = 1, as a dot
+    Dot tol2;
+    if constexpr (F32) {
+        tol2.x = (float)(rtol * rtol);
+        tol2.y = (float)(rtol * rtol - (double)tol2.x);
+        rr = make_float2(1.0f, 0.0f);
+    } else {
+        tol2 = rtol * rtol;
+        rr = 1.0;
+    }
     bool run = !fail && nb2 > 0.0 && isfinite(nb2) && max_iter > 0 && rtol < 1.0;
     if (*sl.bad) run = false, fail = 1;
-    // D^-1 r of slot k (S: its inverse diagonal block): publishes the row, adds to the reduction values
-    auto residual = [&](int m, int k, const T *S, float4 R, T *rm, float v[8], T &d_rr, T &d_rz) {
+    // z = D^-1 r + Z c of slot k with inverse diagonal block S and arm R (zero at an
+    // unused or pinned slot): publishes the row, adds r.z to its dot
+    auto precondition = [&](int m, int k, const T *S, float4 R, const T *rm, Dot &d_rz) {
         T z[D];
+        const int w = __float_as_int(R.w);
         sym_mul<T, D>(S, rm, z);
-        put_row<T, D>(zr(s0 + k), z);
-        float f[D];
+        prolong_add<T, D>(R, scown[one ? 0 : (w & 0xffff) - a0], z);
 #pragma unroll
         for (int c = 0; c < D; ++c) {
+            z[c] = (w >> 30) ? T(0) : z[c];
             if constexpr (KEEP_Z) zk[m][c] = z[c];
-            f[c] = (float)rm[c];
-            d_rr += rm[c] * rm[c];
-            d_rz += rm[c] * z[c];
         }
+        put_row<T, D>(zr(s0 + k), z);
+        dot_add<D, EXACT>(d_rz, rm, z, m == 0);
+    };
+    auto restrict_slot = [&](float4 R, const T *rm, float v[8]) {
+        float f[D];
+#pragma unroll
+        for (int c = 0; c < D; ++c) f[c] = (float)rm[c];
         restrict_to<D>(R, f, v);
     };
     uint32_t tag = 1;
     if (run) {
         const double scale = 1.0 / sqrt(nb2);
         float v[8] = {};
-        T d_rr = T(0), d_rz = T(0);
+        Dot d_rz{};
 #pragma unroll
         for (int m = 0; m < VPT; ++m) {
             const int k = tid + m * nthr;
 #pragma unroll
             for (int c = 0; c < D; ++c) r[m][c] = T(rhs(k, c) * scale);
             if (k < ns) {
-                T S[ND];
-                inv_block(m, k, S);
-                residual(m, k, S, arm(m, k), r[m], v, d_rr, d_rz);
-                if (!one) {
-                    put_sum(m, v);
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) v[q] = 0.0f;
-                }
+                restrict_slot(arm(m, k), r[m], v);
+                if (!one) put_group(m, v);
             }
         }
         if (one) put_sum(0, v);
         if (!exchange(0, nullptr, ss, false, 0, 0, tag)) fail = 1;
         coarse(0.0f, false);
-        // again with the coarse values and r.z
-        if constexpr (F32) {
-            const float t = warp_all((float)d_rz);
-            if (lane == 0) sred[wrp][6] = t;
+        csync(nthr);
+#pragma unroll
+        for (int m = 0; m < VPT; ++m) {
+            const int k = tid + m * nthr;
+            if (k >= ns) continue;
+            T S[ND];
+            inv_block(m, k, S);
+            precondition(m, k, S, arm(m, k), r[m], d_rz);
         }
+        // the same restricted vector again, with r.z and the rows of z
         if (!exchange(1, &d_rz, ss_next, true, 1, 1, tag)) fail = 1;
         swap_s();
-        rz = warp_all(dot_part(1, 0) + coarse_part());
+        dot_sums(1, 1, &rz);
     }
     T beta = T(0);
     while (run && !fail) {
@@ -795,48 +913,31 @@ __device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int ct
         // 1. p = z + beta p at own and halo vertices; A p
 #pragma unroll 2
         for (int h = tid; h < nh; h += nthr) {
-            const int s = shalo[h];
             T z[D], pv[D];
-            get_row<T, D>(zr(s), z);
-            const float4 R = pd.pos4[s];
-            const int w = __float_as_int(R.w);
+            get_row<T, D>(zr(shalo[h]), z);
             ld_vec<T, D>(sp, ns + h, pv);
-            prolong_add<T, D>(R, sc_ + (w & 0xffff) * NM, z);
 #pragma unroll
-            for (int c = 0; c < D; ++c) pv[c] = (w >> 30) ? T(0) : z[c] + beta * pv[c];
+            for (int c = 0; c < D; ++c) pv[c] = z[c] + beta * pv[c];
             st_vec<T, D>(sp, ns + h, pv);
         }
 #pragma unroll
-        for (int m0 = 0; m0 < VPT; m0 += VB) {
-            T z[VB][D];
-            float4 R[VB];
+        for (int m = 0; m < VPT; ++m) {
+            const int k = tid + m * nthr;
+            if (k >= ns) continue;
+            T z[D], pv[D];
+            if constexpr (KEEP_Z) {
 #pragma unroll
-            for (int u = 0; u < VB; ++u) {
-                const int k = tid + (m0 + u) * nthr;
-                if (k >= ns) continue;
-                R[u] = arm(m0 + u, k);
-                if constexpr (KEEP_Z) {
-#pragma unroll
-                    for (int c = 0; c < D; ++c) z[u][c] = zk[m0 + u][c];
-                } else {
-                    get_row<T, D>(zr(s0 + k), z[u]);
-                }
+                for (int c = 0; c < D; ++c) z[c] = zk[m][c];
+            } else {
+                get_row<T, D>(zr(s0 + k), z);
             }
+            ld_vec<T, D>(sp, k, pv);
 #pragma unroll
-            for (int u = 0; u < VB; ++u) {
-                const int k = tid + (m0 + u) * nthr;
-                if (k >= ns) continue;
-                const int w = __float_as_int(R[u].w);
-                T pv[D];
-                ld_vec<T, D>(sp, k, pv);
-                prolong_add<T, D>(R[u], sc_ + (w & 0xffff) * NM, z[u]);
-#pragma unroll
-                for (int c = 0; c < D; ++c) pv[c] = (w >> 30) ? T(0) : z[u][c] + beta * pv[c];
-                st_vec<T, D>(sp, k, pv);
-                if constexpr (!ROWS) {
-                    const T zero[D] = {};
-                    st_vec<T, D>(sy, k, zero);
-                }
+            for (int c = 0; c < D; ++c) pv[c] = z[c] + beta * pv[c];
+            st_vec<T, D>(sp, k, pv);
+            if constexpr (!ROWS) {
+                const T zero[D] = {};
+                st_vec<T, D>(sy, k, zero);
             }
         }
         csync(nthr);
@@ -881,52 +982,33 @@ __device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int ct
         }
         {
             float v[8] = {};
-            T dot = T(0);
+            Dot dot{};
 #pragma unroll
-            for (int m0 = 0; m0 < VPT; m0 += VB) {
-                float4 R[VB];
-                T dh[VB], dy[VB];
+            for (int m = 0; m < VPT; ++m) {
+                const int k = tid + m * nthr;
+                if (k >= ns) continue;
+                const float4 R = arm(m, k);
+                T dh = T(0), dy = T(0);
+                if constexpr (KEEP_S)
+                    dh = dk[m][0], dy = dk[m][1];
+                else if (pd.has_diag)
+                    dh = dg(k)[0], dy = dg(k)[1];
+                float f[D];
+                T pv[D], y[D];
+                const bool fx = (__float_as_int(R.w) >> 30) != 0;
+                ld_vec<T, D>(sp, k, pv);
+                ld_vec<T, D>(sy, k, y);
 #pragma unroll
-                for (int u = 0; u < VB; ++u) {
-                    const int k = tid + (m0 + u) * nthr;
-                    if (k >= ns) continue;
-                    R[u] = arm(m0 + u, k);
-                    dh[u] = dy[u] = T(0);
-                    if constexpr (KEEP_S)
-                        dh[u] = dk[m0 + u][0], dy[u] = dk[m0 + u][1];
-                    else if (pd.has_diag)
-                        dh[u] = dg(k)[0], dy[u] = dg(k)[1];
+                for (int c = 0; c < D; ++c) {
+                    y[c] = fx ? T(0) : y[c] + (c == 1 ? dy : dh) * pv[c];
+                    f[c] = (float)y[c];
                 }
-#pragma unroll
-                for (int u = 0; u < VB; ++u) {
-                    const int k = tid + (m0 + u) * nthr;
-                    if (k >= ns) continue;
-                    float f[D];
-                    T pv[D], y[D];
-                    const bool fx = (__float_as_int(R[u].w) >> 30) != 0;
-                    ld_vec<T, D>(sp, k, pv);
-                    ld_vec<T, D>(sy, k, y);
-#pragma unroll
-                    for (int c = 0; c < D; ++c) {
-                        y[c] = fx ? T(0) : y[c] + (c == 1 ? dy[u] : dh[u]) * pv[c];
-                        f[c] = (float)y[c];
-                        dot += pv[c] * y[c];
-                    }
-                    st_vec<T, D>(sy, k, y);
-                    restrict_to<D>(R[u], f, v);
-                    if (!one) {
-                        if constexpr (F32) v[6] = (float)dot;
-                        put_sum(m0 + u, v);
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) v[q] = 0.0f;
-                        if constexpr (F32) dot = T(0);
-                    }
-                }
+                dot_add<D, EXACT>(dot, pv, y, m == 0);
+                st_vec<T, D>(sy, k, y);
+                restrict_to<D>(R, f, v);
+                if (!one) put_group(m, v);
             }
-            if (one) {
-                if constexpr (F32) v[6] = (float)dot;
-                put_sum(0, v);
-            }
+            if (one) put_sum(0, v);
             if (*sl.bad) {  // a chunk never came: the others give up at their next wait
                 fail = 1;
                 break;
@@ -936,14 +1018,15 @@ __device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int ct
                 break;
             }
         }
-        // 2. alpha; x, r, D^-1 r; the coarse values; r.r and r.z
-        T pAp, alpha;
+        // 2. alpha; x, r; the coarse values; z; r.r and r.z
+        Dot pAp;
+        T alpha;
         if constexpr (F32) {
-            pAp = solo ? sdots[0][0] : warp_all(dot_part(0, 0));
-            alpha = __fdividef(rz, pAp);
+            dot_sums(0, 1, &pAp);
+            alpha = dot_quot(rz, pAp);
         } else {  // one warp forms the FP64 scalars
             if (wrp == 0) {
-                pAp = warp_all(dot_part(0, 0));
+                dot_sums(0, 1, &pAp);
                 if (lane == 0) {
                     sbc[0] = pAp;
                     sbc[1] = rz / pAp;
@@ -953,7 +1036,7 @@ __device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int ct
             pAp = sbc[0];
             alpha = sbc[1];
         }
-        if (!(pAp > T(0)) || !isfinite(pAp)) {
+        if (!(dot_value(pAp) > T(0)) || !isfinite(dot_value(pAp))) {
             neg = 1;
             if (it == 0)  // the preconditioned steepest-descent direction
 #pragma unroll
@@ -966,44 +1049,39 @@ __device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int ct
         coarse((float)alpha, true);
         {
             float v[8] = {};
-            T dots[2] = {T(0), T(0)};
+            Dot dots[2] = {};
+            // x and r go on while some warps form the coarse values; with one slot a thread
+            // (its arm in registers), or two in a CTA of one aggregate, the restriction too
+            constexpr bool EARLY = VPT == 1 || (VPT == 2 && !ROWS);
 #pragma unroll
-            for (int m0 = 0; m0 < VPT; m0 += VB) {
-                T S[VB][ND];
-                float4 R[VB];
+            for (int m = 0; m < VPT; ++m) {
+                const int k = tid + m * nthr;
+                if (k >= ns) continue;
+                T pv[D], y[D];
+                ld_vec<T, D>(sp, k, pv);
+                ld_vec<T, D>(sy, k, y);
 #pragma unroll
-                for (int u = 0; u < VB; ++u) {
-                    const int k = tid + (m0 + u) * nthr;
-                    if (k >= ns) continue;
-                    R[u] = arm(m0 + u, k);
-                    inv_block(m0 + u, k, S[u]);
+                for (int c = 0; c < D; ++c) {
+                    x[m][c] += alpha * pv[c];
+                    r[m][c] -= alpha * y[c];
                 }
-#pragma unroll
-                for (int u = 0; u < VB; ++u) {
-                    const int m = m0 + u, k = tid + m * nthr;
-                    if (k >= ns) continue;
-                    T pv[D], y[D];
-                    ld_vec<T, D>(sp, k, pv);
-                    ld_vec<T, D>(sy, k, y);
-#pragma unroll
-                    for (int c = 0; c < D; ++c) {
-                        x[m][c] += alpha * pv[c];
-                        r[m][c] -= alpha * y[c];
-                    }
-                    residual(m, k, S[u], R[u], r[m], v, dots[0], dots[1]);
-                    if (!one) {
-                        if constexpr (F32) v[6] = (float)dots[0], v[7] = (float)dots[1];
-                        put_sum(m, v);
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) v[q] = 0.0f;
-                        if constexpr (F32) dots[0] = dots[1] = T(0);
-                    }
-                }
+                dot_add<D, EXACT>(dots[0], r[m], r[m], m == 0);
+                if (EARLY) restrict_slot(arm(m, k), r[m], v);
             }
-            if (one) {
-                if constexpr (F32) v[6] = (float)dots[0], v[7] = (float)dots[1];
-                put_sum(0, v);
+            if (EARLY) put_sum(0, v);
+            csync(nthr);
+#pragma unroll
+            for (int m = 0; m < VPT; ++m) {
+                const int k = tid + m * nthr;
+                if (k >= ns) continue;
+                const float4 R = arm(m, k);
+                T S[ND];
+                inv_block(m, k, S);
+                if (!EARLY) restrict_slot(R, r[m], v);
+                precondition(m, k, S, R, r[m], dots[1]);
+                if (!EARLY && !one) put_group(m, v);
             }
+            if (!EARLY && one) put_sum(0, v);
             if (!exchange(2, dots, ss_next, true, 1, 1, tag)) {
                 fail = 1;
                 break;
@@ -1011,23 +1089,22 @@ __device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int ct
             swap_s();
         }
         ++it;
-        T rz_new;
-        if (F32 || wrp == 0) {
-            rr = dot_part(1, 0);
-            rz_new = dot_part(1, 1) + coarse_part();
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                rr += __shfl_xor_sync(0xffffffffu, rr, o);
-                rz_new += __shfl_xor_sync(0xffffffffu, rz_new, o);
-            }
-        }
+        Dot rz_new;
         if constexpr (F32) {
-            beta = __fdividef(rz_new, rz);
+            Dot two[2];
+            dot_sums(1, 2, two);
+            rr = two[0];
+            rz_new = two[1];
+            beta = dot_quot(rz_new, rz);
         } else {
-            if (wrp == 0 && lane == 0) {
-                sbc[0] = rr;
-                sbc[1] = rz_new;
-                sbc[2] = rz_new / rz;
+            if (wrp == 0) {
+                Dot two[2];
+                dot_sums(1, 2, two);
+                if (lane == 0) {
+                    sbc[0] = two[0];
+                    sbc[1] = two[1];
+                    sbc[2] = two[1] / rz;
+                }
             }
             csync(nthr);
             rr = sbc[0];
@@ -1035,7 +1112,7 @@ __device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int ct
             beta = sbc[2];
         }
         rz = rz_new;
-        if (!(rr > tol2) || it >= max_iter || !isfinite(rr) || !(rz > T(0))) break;
+        if (!(dot_minus(rr, tol2) > T(0)) || it >= max_iter || !isfinite(dot_value(rr)) || !(dot_value(rz) > T(0))) break;
     }
     const double bnorm = nb2 > 0.0 && isfinite(nb2) ? sqrt(nb2) : 0.0;
 #pragma unroll
@@ -1049,7 +1126,10 @@ __device__ __forceinline__ PcgResult pcg_run(const PcgDev &pd, Slice &sl, int ct
     res.iter = it;
     res.neg = neg;
     res.fail = fail;
-    res.rr = (double)rr * bnorm * bnorm;
+    if constexpr (F32)
+        res.rr = ((double)rr.x + (double)rr.y) * bnorm * bnorm;
+    else
+        res.rr = rr * bnorm * bnorm;
     return res;
 }
 

@@ -22,11 +22,17 @@
 // each edge once, streamed every iteration by a producer warp through a ring of
 // bulk copies that runs ahead across the barriers.  Two exchanges between the
 // CTAs an iteration:
-//   1. p = z + beta p at own and halo vertices (z from the published D^-1 r
-//      and the coarse vector); A p; p.Ap and Z^T A p; exchange;
-//   2. alpha; x, r, D^-1 r (published); the coarse vector of the new residual
-//      from E^-1 (Z^T r - alpha Z^T A p), so it is ready before the exchange;
-//      r.r, r.D^-1 r, the new Z^T r; exchange; beta and the convergence test.
+//   1. p = z + beta p at own and halo vertices (z as published); A p; p.Ap and
+//      Z^T A p; exchange;
+//   2. alpha; x, r; the coarse values of the CTA's own aggregates for the new
+//      residual from E^-1 (Z^T r - alpha Z^T A p), so z is whole before the
+//      exchange; z (published); r.r, r.z, the new Z^T r; exchange; beta and the
+//      convergence test.
+// The dots are formed from the vectors themselves, compensated pairs in FP32 and
+// FP64 else, through threads, warps and CTAs up to the quotients alpha and
+// beta: the first step length is within 7e-8 of its value in 64 bits (FP32's own
+// rounding; 1.2e-7 to 2.2e-7 with plain FP32 sums), on FP64 handles within 4e-16
+// (5e-8 with the coarse share of r.z from the FP32 restriction).
 // An exchange is barrier and data in one: on a grid every CTA stores its sums
 // as (value, tag) words and polls the words of all CTAs; in a cluster it pushes
 // them into the other CTAs' shared memory before the hardware barrier.  Every
@@ -46,8 +52,9 @@ namespace {
 constexpr int kPcgThreads = 512;
 }
 
-// ROWS: the slices are stored by rows (see cg_plan.h), else by colours.
-template <typename T, int D, int VPT, bool ROWS>
+// ROWS: the slices are stored by rows (see cg_plan.h), else by colours.  GRID: a
+// cooperative grid, else one CTA or one cluster.
+template <typename T, int D, int VPT, bool ROWS, bool GRID>
 __global__ void __launch_bounds__(512, 1)
     k_pcg(PcgDev pd, const double *__restrict__ b, double sign, T *__restrict__ dout, double rtol, int max_iter,
           int polls, DevScalars *sc)
@@ -56,7 +63,7 @@ __global__ void __launch_bounds__(512, 1)
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int sbad, sstop;
     const int cta = blockIdx.x, nthr = pd.threads, tid = threadIdx.x, lane = tid & 31;
-    const bool grid = pd.n_cta > 1 && !pd.cluster;
+    constexpr bool grid = GRID;
     Slice sl = pcg_slice<D, T, ROWS>(pd, cta, grid, smem, polls, &sbad);
     const unsigned char *gsl = sl.rest - sl.n_ent * esz;  // this CTA's slice in global memory
     if (tid == 0) {
@@ -111,7 +118,7 @@ __global__ void __launch_bounds__(512, 1)
         csync(nthr);
         const int bad = sbad;
         int any = bad;
-        if (pd.cluster) {  // the CTAs of a cluster leave together or not at all
+        if (!GRID && pd.cluster) {  // the CTAs of a cluster leave together or not at all
             cluster_sync();
             for (int k = 0; k < pd.n_cta; ++k) any |= ld_dsmem_s32(&sbad, (uint32_t)k);
             cluster_sync();
@@ -125,12 +132,12 @@ __global__ void __launch_bounds__(512, 1)
         }
     }
     const PcgResult res =
-        pcg_run<T, D, VPT, ROWS>(pd, sl, cta, grid, smem, b, sign, sc->gn2, dout, rtol, max_iter, true);
+        pcg_run<T, D, VPT, ROWS, GRID>(pd, sl, cta, smem, b, sign, sc->gn2, dout, rtol, max_iter, true);
     if (sl.stages) {
         csync(nthr);
         if (tid == 0) *(volatile int *)&sstop = 1;
     }
-    if (pd.cluster) cluster_sync();  // no CTA leaves while another may still write to it
+    if (!GRID && pd.cluster) cluster_sync();  // no CTA leaves while another may still write to it
     if (res.fail && tid == 0) atomicOr(&sc->kerr, sbad ? 1 : 2);
     if (cta == 0 && tid == 0) {
         sc->iter = res.iter;
@@ -143,16 +150,21 @@ __global__ void __launch_bounds__(512, 1)
 // ---------------------------------------------------------------- host side
 
 template <typename T, int D>
-static void *pcg_kernel(int vpt, bool rows)
+static void *pcg_kernel(const PcgDev &pd)
 {
-    if (rows) return vpt == 1 ? (void *)k_pcg<T, D, 1, true> : (void *)k_pcg<T, D, 4, true>;
-    switch (vpt) {
-        case 1: return (void *)k_pcg<T, D, 1, false>;
-        case 2: return (void *)k_pcg<T, D, 2, false>;
-        case 4: return (void *)k_pcg<T, D, 4, false>;
+    const bool grid = pd.n_cta > 1 && !pd.cluster;
+    if (pd.tpr) {
+        if (grid) return pd.vpt == 1 ? (void *)k_pcg<T, D, 1, true, true> : (void *)k_pcg<T, D, 4, true, true>;
+        return pd.vpt == 1 ? (void *)k_pcg<T, D, 1, true, false> : (void *)k_pcg<T, D, 4, true, false>;
+    }
+    if (!grid) return nullptr;  // parts of one CTA or a cluster are stored by rows
+    switch (pd.vpt) {
+        case 1: return (void *)k_pcg<T, D, 1, false, true>;
+        case 2: return (void *)k_pcg<T, D, 2, false, true>;
+        case 4: return (void *)k_pcg<T, D, 4, false, true>;
         default:
             if constexpr (sizeof(T) == 4)
-                return (void *)k_pcg<T, D, 8, false>;
+                return (void *)k_pcg<T, D, 8, false, true>;
             else
                 return nullptr;  // x and r would not fit in the registers
     }
@@ -208,7 +220,7 @@ static bool configure(const Ctx &c, PcgDev &pd)
     const size_t esz = 4 + D * D * sizeof(T);
     const bool on_grid = pd.n_cta > 1 && !pd.cluster;
     const PcgSmem base(D, sizeof(T), pd.ns, pd.max_halo, pd.max_items, pd.n_coarse, pd.n_meta, on_grid ? pd.n_cta : 0);
-    if (pd.max_items > (on_grid ? 1 : kMaxWarps)) return false;
+    if (pd.max_items > (on_grid ? 1 : kMaxWarps) || pd.n_cta > 32 * kMaxWarps) return false;
     const bool rows = pd.tpr > 0;
     for (int streamed = 0; streamed < (rows ? 1 : 2); ++streamed) {
         // 512 threads with 128 registers each: a producer warp takes one warp's place
@@ -218,9 +230,9 @@ static bool configure(const Ctx &c, PcgDev &pd)
         const int need = (pd.ns + pd.threads - 1) / pd.threads;
         if (need > (sizeof(T) == 8 || rows ? 4 : 8)) return false;
         pd.vpt = need <= 1 ? 1 : need <= 2 && !rows ? 2 : need <= 4 ? 4 : 8;
-        void *k = pcg_kernel<T, D>(pd.vpt, rows);
+        void *k = pcg_kernel<T, D>(pd);
         cudaFuncAttributes at;
-        if (cudaFuncGetAttributes(&at, k) != cudaSuccess) break;
+        if (!k || cudaFuncGetAttributes(&at, k) != cudaSuccess) break;
         // every handle sets the same limit: attributes belong to the function, not to a handle
         const size_t limit = kPcgSmem - at.sharedSizeBytes;
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit) != cudaSuccess ||
@@ -254,7 +266,7 @@ template <typename T>
 cudaError_t launch_pcg(const Ctx &c, const PcgDev &pd, const double *b, double sign, T *d, double rtol, int max_iter,
                        cudaStream_t s)
 {
-    void *k = c.dim == 2 ? pcg_kernel<T, 2>(pd.vpt, pd.tpr > 0) : pcg_kernel<T, 3>(pd.vpt, pd.tpr > 0);
+    void *k = c.dim == 2 ? pcg_kernel<T, 2>(pd) : pcg_kernel<T, 3>(pd);
     int polls = c.td.wait_polls;
     DevScalars *sc = c.sc;
     void *args[] = {(void *)&pd, (void *)&b, &sign, &d, &rtol, &max_iter, &polls, &sc};

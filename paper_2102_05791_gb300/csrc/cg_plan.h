@@ -46,8 +46,11 @@ constexpr uint32_t kCgLastOfColour = 0x80000000u;
 constexpr uint32_t kCgTransposed = 0x80000000u;
 constexpr int kPcgMaxStages = 8;
 constexpr int kPcgSmem = 226 * 1024;     // shared memory of one CTA, static part included
-constexpr int kPcgStatic = 10 * 1024;     // room for the kernels' static part when a slice is sized
-constexpr int kPcgWords = 18;            // words of a CTA in a grid's exchange: items from 0, coarse values from 8, dots from 14
+constexpr int kPcgStatic = 12 * 1024;     // room for the kernels' static part when a slice is sized
+// Words of a CTA in a grid's exchange: items from 0, two words a dot from kPcgDots; in
+// memory a 128-byte line (80 bytes, sharing lines: 0.2 to 1.1 us an iteration more), in
+// shared memory rows that spread over the banks.
+constexpr int kPcgWords = 16, kPcgRow = 18, kPcgDots = 6;
 constexpr int kCgMaxCoarse = 192;  // coarse unknowns (cg_assemble.cu inverts the coarse matrix in one CTA's registers)
 constexpr int kCgCoarseItem = 1024;  // edges or slots per partial sum of the coarse matrix
 
@@ -56,7 +59,7 @@ enum CoarseKind { CK_INNER = 0, CK_CROSS = 1, CK_LO = 2, CK_HI = 3, CK_VERT = 4 
 
 // Shared-memory plan of the solver (byte offsets; the edge slice or ring starts at ring).
 struct PcgSmem {
-    size_t p, y, e, c, s, t, meta, halo, word, ring;
+    size_t p, y, e, s, t, meta, halo, word, ring;
 #ifdef __CUDACC__
     __host__ __device__
 #endif
@@ -66,13 +69,12 @@ struct PcgSmem {
         y = p + (size_t)(ns + max_halo) * dim * elt;
         e = y + (size_t)ns * dim * elt;
         e = (e + 15) / 16 * 16;
-        c = e + (size_t)items * (dim == 3 ? 6 : 3) * n_coarse * 4;
-        s = c + (size_t)n_coarse * 4;
+        s = e + (size_t)items * (dim == 3 ? 6 : 3) * n_coarse * 4;
         t = s + (size_t)n_coarse * 8;  // two buffers
         meta = t + (size_t)n_coarse * 4;
         halo = meta + (size_t)n_meta * 4;
-        word = halo + (size_t)max_halo * 4;
-        ring = (word + (size_t)grid_ctas * kPcgWords * 4 + 127) / 128 * 128;
+        word = (halo + (size_t)max_halo * 4 + 7) / 8 * 8;
+        ring = (word + (size_t)grid_ctas * kPcgRow * 4 + 127) / 128 * 128;
     }
 };
 
