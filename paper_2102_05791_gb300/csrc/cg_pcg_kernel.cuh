@@ -48,10 +48,6 @@
 
 namespace softsim {
 
-namespace {
-constexpr int kPcgThreads = 512;
-}
-
 // ROWS: the slices are stored by rows (see cg_plan.h), else by colours.  GRID: a
 // cooperative grid, else one CTA or one cluster.
 template <typename T, int D, int VPT, bool ROWS, bool GRID>
@@ -223,12 +219,12 @@ static bool configure(const Ctx &c, PcgDev &pd)
     if (pd.max_items > (on_grid ? 1 : kMaxWarps) || pd.n_cta > 32 * kMaxWarps) return false;
     const bool rows = pd.tpr > 0;
     for (int streamed = 0; streamed < (rows ? 1 : 2); ++streamed) {
-        // 512 threads with 128 registers each: a producer warp takes one warp's place
-        pd.threads = streamed ? kPcgThreads - 32
+        // a producer warp takes one warp's place
+        pd.threads = streamed ? kPcgStreamThreads
                      : rows   ? std::min(kPcgThreads, std::max(128, pd.ns * pd.tpr))
                      : kPcgThreads;
         const int need = (pd.ns + pd.threads - 1) / pd.threads;
-        if (need > (sizeof(T) == 8 || rows ? 4 : 8)) return false;
+        if (need > pcg_max_vpt(sizeof(T), rows)) return false;
         pd.vpt = need <= 1 ? 1 : need <= 2 && !rows ? 2 : need <= 4 ? 4 : 8;
         void *k = pcg_kernel<T, D>(pd);
         cudaFuncAttributes at;

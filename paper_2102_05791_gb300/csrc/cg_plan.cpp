@@ -121,6 +121,36 @@ int aggregates_per_part(int64_t v, int most, int threads)
     return best;
 }
 
+// Parts (CTAs), aggregates and storage of the persistent CG solver for a mesh
+// of nv vertices.  The lines lie where both sides measured alike (microseconds
+// an iteration on GB300): one cluster exchanges in about 1 us, a grid in about
+// 2 us, so a cluster's 16 CTAs serve as long as their rows stay in shared
+// memory (3D FP32: 4.7 us at 1,260 vertices; 7.9 on a grid of 64 at 9,537, where
+// 16 CTAs need 18; 2D: 7.2 at 20,000).  FP64 arithmetic is scarce, so FP64
+// spreads over more CTAs earlier (16.0 us on 64 CTAs against 18.8 on 16 at 2,640
+// vertices).  More aggregates save iterations but cost a larger inverse (192
+// coarse unknowns: 0.12 ms, 96: 0.02 ms), which small meshes do not win back.
+// Rows beat colours until the part's rows no longer stay in L2 (3D FP32: 23.4
+// against 22.9 us at 122,000 vertices, 42.8 against 30.9 at 180,000).
+PcgSizes pcg_sizes(int dim, int elt, int64_t nv, int n_sm)
+{
+    const bool f32 = elt == 4;
+    const int nm = dim == 3 ? 6 : 3;
+    const int64_t per_cta = dim == 3 ? (f32 ? 270 : 100) : (f32 ? 1300 : 256);  // the most a cluster's CTA takes
+    int64_t g, a = std::max<int64_t>(1, std::min<int64_t>((nv <= 4096 ? kCgMaxCoarse / 2 : kCgMaxCoarse) / nm, nv / 18));
+    if (nv <= 16 * per_cta) {
+        g = f32 && nv <= 160 ? 1 : std::min<int64_t>(16, (nv + 31) / 32);
+        a = std::min(a, 16 * g);
+    } else {
+        g = std::min<int64_t>(n_sm, std::max<int64_t>(kCgMaxCoarse / nm, nv / (dim == 3 ? (f32 ? 150 : 40) : 256)));
+        a = std::min(a, g);
+    }
+    const int64_t per = (nv + g - 1) / g;
+    if (a > g) a = g * aggregates_per_part(per, (int)(a / g), 512);
+    const bool rows = per <= (dim == 3 ? (f32 ? 750 : 600) : 2000);
+    return {(int)g, (int)a, g > 1 && g <= 16, rows, per <= (int64_t)pcg_max_vpt(elt, rows) * kPcgStreamThreads};
+}
+
 bool batch_plan_fits(const CgPlan &P, int threads)
 {
     const size_t N = (size_t)P.n_agg * P.n_modes, esz = 4 + (size_t)P.dim * P.dim * sizeof(float);
@@ -147,6 +177,10 @@ bool build_cg_plan(int dim, int64_t nv, int64_t ne, const double *X, const int32
     const int n_parts = n_cta * per;
     if (nv < n_parts || n_agg < 1) {
         err = "fewer vertices than parts";
+        return false;
+    }
+    if (ne > INT32_MAX / nc) {  // the incidences are counted in 32 bits
+        err = "too many elements";
         return false;
     }
 

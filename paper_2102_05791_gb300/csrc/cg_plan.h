@@ -45,6 +45,8 @@ constexpr uint32_t kCgPadEntry = 0xffffffffu;
 constexpr uint32_t kCgLastOfColour = 0x80000000u;
 constexpr uint32_t kCgTransposed = 0x80000000u;
 constexpr int kPcgMaxStages = 8;
+constexpr int kPcgThreads = 512;          // threads of a CTA at most (128 registers each)
+constexpr int kPcgStreamThreads = kPcgThreads - 32;  // beside the producer warp of a streamed slice
 constexpr int kPcgSmem = 226 * 1024;     // shared memory of one CTA, static part included
 constexpr int kPcgStatic = 12 * 1024;     // room for the kernels' static part when a slice is sized
 // Words of a CTA in a grid's exchange: items from 0, two words a dot from kPcgDots; in
@@ -121,6 +123,18 @@ struct CgPlan {
 // keeps to `threads` slots (one a thread) or wastes less than a fifth of the
 // slots, else the least wasteful.
 int aggregates_per_part(int64_t v, int most, int threads);
+
+// Slots of a thread at most: x and r of a slot stay in its registers.
+inline int pcg_max_vpt(int elt, bool rows) { return elt == 8 || rows ? 4 : 8; }
+
+// Parts (CTAs), aggregates and storage of the persistent solver for a mesh of nv
+// vertices; fits: a CTA's threads can hold its vertices (a part is streamed at
+// the limit, by kPcgStreamThreads threads).
+struct PcgSizes {
+    int n_cta, n_agg;
+    bool cluster, rows, fits;
+};
+PcgSizes pcg_sizes(int dim, int elt, int64_t nv, int n_sm);
 
 // The batched solver: dynamic shared memory of the plan's layout (the body's
 // plan record lies behind it), and vertices of a body per thread at most.

@@ -393,9 +393,14 @@ static int create_impl(sim_handle *h, const sim_mesh *mesh, const sim_material *
     c.vd.X = h->X;
     c.vd.mass = h->mass;
     c.vd.fixed = h->fixed;
+    CK(h, cudaDeviceGetAttribute(&h->n_sm, cudaDevAttrMultiProcessorCount, h->device));
     if (h->opt.cg_kernel == SIM_CG_AUTO) {
-        h->rest.assign(mesh->rest_pos, mesh->rest_pos + nv * d);
-        h->elems.assign(mesh->elems, mesh->elems + ne * nc);
+        if (pcg_sizes(d, is_mixed(h) ? 4 : 8, nv, h->n_sm).fits) {
+            h->rest.assign(mesh->rest_pos, mesh->rest_pos + nv * d);
+            h->elems.assign(mesh->elems, mesh->elems + ne * nc);
+        } else {  // known without building the plan (0.6 s and more at these sizes)
+            h->pcg_state = -1;
+        }
     }
     TileDev &td = c.td;
     td.n_tiles = tb.n_tiles;
@@ -446,7 +451,6 @@ static int create_impl(sim_handle *h, const sim_mesh *mesh, const sim_material *
     c.muscle = h->mat.muscle_model;
     if (c.threads % 32 || c.threads > 256) return fail(h, SIM_EINVAL, "threads must be a multiple of 32, at most 256");
     c.n_fin_blocks = std::max(1, (td.n_fin + 255) / 256);
-    CK(h, cudaDeviceGetAttribute(&h->n_sm, cudaDevAttrMultiProcessorCount, h->device));
     c.split = eval_split(td.n_tiles, h->n_sm);
     // element kernel of the assembly: warps for every SM, one element a thread at most
     c.asm_split = std::min((td.max_te + c.threads - 1) / c.threads, std::max(1, 8 * h->n_sm / td.n_tiles));
@@ -686,43 +690,11 @@ static cudaGraphExec_t get_cg_while(sim_handle *h, const Phys &ph)
 // Rounds of the device-side loop that cover max_iter iterations, plus slack.
 static int cg_max_rounds(int max_iter) { return max_iter / kCgBody + 2; }
 
-// Parts (CTAs), aggregates and storage of the persistent CG solver for a mesh
-// of nv vertices.  The lines lie where both sides measured alike (microseconds
-// an iteration on GB300): one cluster exchanges in about 1 us, a grid in about
-// 2 us, so a cluster's 16 CTAs serve as long as their rows stay in shared
-// memory (3D FP32: 4.7 us at 1,260 vertices; 7.9 on a grid of 64 at 9,537, where
-// 16 CTAs need 18; 2D: 7.2 at 20,000).  FP64 arithmetic is scarce, so FP64
-// spreads over more CTAs earlier (16.0 us on 64 CTAs against 18.8 on 16 at 2,640
-// vertices).  More aggregates save iterations but cost a larger inverse (192
-// coarse unknowns: 0.12 ms, 96: 0.02 ms), which small meshes do not win back.
-// Rows beat colours until the part's rows no longer stay in L2 (3D FP32: 23.4
-// against 22.9 us at 122,000 vertices, 42.8 against 30.9 at 180,000).
-struct PcgSizes {
-    int n_cta, n_agg;
-    bool cluster, rows;
-};
-static PcgSizes pcg_sizes(int dim, bool f32, int64_t nv, int n_sm)
-{
-    const int nm = dim == 3 ? 6 : 3;
-    const int64_t per_cta = dim == 3 ? (f32 ? 270 : 100) : (f32 ? 1300 : 256);  // the most a cluster's CTA takes
-    int64_t g, a = std::max<int64_t>(1, std::min<int64_t>((nv <= 4096 ? kCgMaxCoarse / 2 : kCgMaxCoarse) / nm, nv / 18));
-    if (nv <= 16 * per_cta) {
-        g = f32 && nv <= 160 ? 1 : std::min<int64_t>(16, (nv + 31) / 32);
-        a = std::min(a, 16 * g);
-    } else {
-        g = std::min<int64_t>(n_sm, std::max<int64_t>(kCgMaxCoarse / nm, nv / (dim == 3 ? (f32 ? 150 : 40) : 256)));
-        a = std::min(a, g);
-    }
-    const int64_t per = (nv + g - 1) / g;
-    if (a > g) a = g * aggregates_per_part(per, (int)(a / g), 512);
-    return {(int)g, (int)a, g > 1 && g <= 16, per <= (dim == 3 ? (f32 ? 750 : 600) : 2000)};
-}
-
 template <typename T>
 static int build_pcg(sim_handle *h, cudaStream_t s)
 {
     int rc;
-    const PcgSizes z = pcg_sizes(h->dim, sizeof(T) == 4, h->nv, h->n_sm);
+    const PcgSizes z = pcg_sizes(h->dim, sizeof(T), h->nv, h->n_sm);
     CgPlan P;
     std::string err;
     h->pcg_state = -1;
