@@ -500,6 +500,8 @@ static int create_impl(sim_handle *h, const sim_mesh *mesh, const sim_material *
         CK(h, cudaMemset(h->u0, 0, sizeof(double) * nd));
     }
     CK(h, cudaMemset(h->vp, 0, vbytes * nd));
+    CK(h, cudaMemset(c.a64, 0, sizeof(double) * ne_int));  // sim_time_hvp reads them, perhaps before any solve
+    if (c.a32) CK(h, cudaMemset(c.a32, 0, sizeof(float) * ne_int));
     if (h->u32) CK(h, cudaMemset(h->u32, 0, sizeof(float) * nd));
     CK(h, cudaMallocHost((void **)&h->sc_host, sizeof(DevScalars)));
     CK(h, cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking));
