@@ -148,22 +148,21 @@ __global__ void __launch_bounds__(512, 1)
 template <typename T, int D>
 static void *pcg_kernel(const PcgDev &pd)
 {
+    constexpr bool F32 = sizeof(T) == 4;
     const bool grid = pd.n_cta > 1 && !pd.cluster;
     if (pd.tpr) {
-        if (grid) return pd.vpt == 1 ? (void *)k_pcg<T, D, 1, true, true> : (void *)k_pcg<T, D, 4, true, true>;
-        return pd.vpt == 1 ? (void *)k_pcg<T, D, 1, true, false> : (void *)k_pcg<T, D, 4, true, false>;
+        if (pd.vpt == 1) return grid ? (void *)k_pcg<T, D, 1, true, true> : (void *)k_pcg<T, D, 1, true, false>;
+        if (grid) return (void *)k_pcg<T, D, 4, true, true>;
+        if constexpr (F32 && D == 2) return (void *)k_pcg<T, D, 4, true, false>;
+    } else {
+        if constexpr (D == 3)
+            if (pd.vpt == 2) return (void *)k_pcg<T, D, 2, false, true>;
+        if constexpr (F32 || D == 3)
+            if (pd.vpt == 4) return (void *)k_pcg<T, D, 4, false, true>;
+        if constexpr (F32)
+            if (pd.vpt == 8) return (void *)k_pcg<T, D, 8, false, true>;
     }
-    if (!grid) return nullptr;  // parts of one CTA or a cluster are stored by rows
-    switch (pd.vpt) {
-        case 1: return (void *)k_pcg<T, D, 1, false, true>;
-        case 2: return (void *)k_pcg<T, D, 2, false, true>;
-        case 4: return (void *)k_pcg<T, D, 4, false, true>;
-        default:
-            if constexpr (sizeof(T) == 4)
-                return (void *)k_pcg<T, D, 8, false, true>;
-            else
-                return nullptr;  // x and r would not fit in the registers
-    }
+    return nullptr;
 }
 
 // The launch of a configured plan, in place; at[1] is filled in too.
@@ -224,8 +223,8 @@ static bool configure(const Ctx &c, PcgDev &pd)
                      : rows   ? std::min(kPcgThreads, std::max(128, pd.ns * pd.tpr))
                      : kPcgThreads;
         const int need = (pd.ns + pd.threads - 1) / pd.threads;
-        if (need > pcg_max_vpt(sizeof(T), rows)) return false;
-        pd.vpt = need <= 1 ? 1 : need <= 2 && !rows ? 2 : need <= 4 ? 4 : 8;
+        pd.vpt = pcg_variant(D, sizeof(T), rows, on_grid, need);
+        if (!pd.vpt) return false;
         void *k = pcg_kernel<T, D>(pd);
         cudaFuncAttributes at;
         if (!k || cudaFuncGetAttributes(&at, k) != cudaSuccess) break;

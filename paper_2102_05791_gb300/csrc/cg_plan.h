@@ -127,6 +127,19 @@ int aggregates_per_part(int64_t v, int most, int threads);
 // Slots of a thread at most: x and r of a slot stay in its registers.
 inline int pcg_max_vpt(int elt, bool rows) { return elt == 8 || rows ? 4 : 8; }
 
+// Slots a thread of the kernel variant that serves `need` of them, 0 if there is
+// none.  One CTA and clusters store by rows and, but for 2D FP32, never have more
+// slots than threads; parts stored by colours have more than 600 vertices in 3D and
+// more than 2,000 in 2D, which FP64 does not reach (pcg_sizes).
+inline int pcg_variant(int dim, int elt, bool rows, bool grid, int need)
+{
+    const int few = rows ? 1 : dim == 3 ? 2 : 4;
+    const int most = rows ? (grid || (dim == 2 && elt == 4) ? 4 : 1) : !grid || (dim == 2 && elt == 8) ? 0 : pcg_max_vpt(elt, false);
+    if (need > most) return 0;
+    if (need <= few) return few;
+    return need <= 4 ? 4 : 8;
+}
+
 // Parts (CTAs), aggregates and storage of the persistent solver for a mesh of nv
 // vertices; fits: a CTA's threads can hold its vertices (a part is streamed at
 // the limit, by kPcgStreamThreads threads).
