@@ -41,7 +41,7 @@ static void bisect(int dim, const double *X, int32_t *ids, int64_t n, const int 
     if (depth > 0 && n > 20000) {
         try {
             t = std::thread([&]() { bisect(dim, X, ids, m, w, left, base, cut, depth - 1); });
-        } catch (const std::system_error &) {  // this thread does both halves
+        } catch (...) {  // no thread, or no memory to start one: this thread does both halves
         }
     }
     const bool both = !t.joinable();

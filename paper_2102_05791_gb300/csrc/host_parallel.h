@@ -5,7 +5,6 @@
 #include <atomic>
 #include <cstdint>
 #include <new>
-#include <system_error>
 #include <thread>
 #include <vector>
 
@@ -35,7 +34,7 @@ void parallel_for(int64_t work_size, int64_t n, int64_t block, F f)
     th.reserve(n_thr);
     try {
         for (int t = 1; t < n_thr; ++t) th.emplace_back(work);
-    } catch (const std::system_error &) {  // fewer threads do
+    } catch (...) {  // no thread, or no memory to start one: fewer threads do
     }
     work();
     for (auto &t : th) t.join();

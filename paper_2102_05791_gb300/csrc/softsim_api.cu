@@ -752,6 +752,8 @@ static int use_pcg(sim_handle *h, bool *use, cudaStream_t s)
             rc = build_pcg<T>(h, s);
         } catch (const std::exception &) {  // no host memory for the plan: per-iteration kernels
             h->pcg_state = -1;
+            std::vector<double>().swap(h->rest);
+            std::vector<int32_t>().swap(h->elems);
         }
         if (rc) return rc;
     }
