@@ -310,7 +310,7 @@ def run_accuracy_quasistatic(dev, name):
 
 
 def run_dot_accuracy(sim, sim64, x, a, dev):
-    """The mixed CG loop's p.Ap (FP32 element quadratic forms, FP32 sums within
+    """The per-iteration mixed CG loop's p.Ap (FP32 element quadratic forms, FP32 sums within
     a tile, compensated sums over the tiles) against the FP64 handle's v.(H v)
     at the same state and direction (the FP64 kernels match the oracle to
     1e-12 of the contribution scale)."""
@@ -713,8 +713,8 @@ def run_ours(args, rank, world, local_rank):
         "higher_is_better": True,
         "scaling": "weak",
         "vs_baseline": None,
-        "dtype": ("f32 HVP and CG vectors; CG dot products f32 within a tile or block and compensated f32 across "
-                  "them; f64 state, gradient, energies, line search and residual checks")
+        "dtype": ("f32 CG operator and vectors; compensated f32 CG dot products; f64 state, gradient, energies, "
+                  "line search and residual checks")
                  if args.precision == "mixed" else "f64",
         "data": "synthetic",
         "config": {"workload": desc, "precision": args.precision,

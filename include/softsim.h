@@ -104,9 +104,11 @@ typedef struct {
 } sim_material;
 
 typedef struct {
-    int precision;            /* SIM_PREC_FP64 (all FP64) or SIM_PREC_MIXED
-                                 (FP32 HVP and CG vectors; FP64 state, gradient,
-                                 energy, reductions and residual checks) */
+    int precision;            /* SIM_PREC_FP64 (all FP64, but for the coarse part of
+                                 the persistent CG solver's preconditioner) or
+                                 SIM_PREC_MIXED (FP32 HVP and CG vectors, CG dot
+                                 products in compensated FP32; FP64 state, gradient,
+                                 energy, their reductions and residual checks) */
     double newton_rtol;       /* stop when |grad| <= newton_rtol |grad_0| */
     double newton_forcing;    /* cap of the CG forcing term: each Newton step's CG
                                  stops at |r| <= min(newton_forcing,
@@ -128,7 +130,9 @@ typedef struct {
                                  kernels;
                                  SIM_CG_ITERATION: always per-iteration kernels,
                                  matrix-free and without preconditioner.  The plan of
-                                 the persistent solver is built by the first solve */
+                                 the persistent solver is built by the first solve and
+                                 takes device memory then, 380 to 480 bytes a tet
+                                 (mixed); without it the per-iteration kernels run */
 } sim_options;
 
 typedef struct {
@@ -176,8 +180,8 @@ int sim_energy_grad(sim_handle *h, const double *x, const double *a, double *E_d
 int sim_hvp(sim_handle *h, const double *x, const double *a, const void *v, void *Hv,
             void *stream);
 
-/* The CG loop's inner product v.(H v) (Eq. matrix-free-dfdx), formed as the
- * CG loop forms p.Ap: each element's quadratic form v_e.(H_e v_e) plus the
+/* The inner product v.(H v) (Eq. matrix-free-dfdx), formed as the
+ * per-iteration CG loop (SIM_CG_ITERATION) forms p.Ap: each element's quadratic form v_e.(H_e v_e) plus the
  * per-vertex terms, summed in FP32 within a tile and with compensated FP32
  * over the tiles (SIM_PREC_MIXED), or in FP64 throughout (SIM_PREC_FP64).
  * Diagnostic, to measure that sum's error.  v, Hv: DEVICE [n_vert][dim] in
@@ -308,8 +312,10 @@ int sim_tile_stats(const sim_handle *h, int *n_tiles, double *elems_per_tile,
  * per step) and backward pass (refined adjoint CG and parameter VJP per step,
  * Eq. dLda-re-ordered) with block- or cluster-level synchronisation only.
  * Mixed precision as SIM_PREC_MIXED.  Deterministic: the number of CTAs and
- * threads of a mesh is fixed when the batch is created, its sums have a fixed
- * order. */
+ * threads of a mesh is fixed when the batch is created (it depends on the
+ * batch's other meshes and the GPU, and so do the last bits), its sums have a
+ * fixed order.  Meshes whose CG plan does not fit, or all when the device has no
+ * memory for the plans, are solved matrix-free. */
 typedef struct sim_batch sim_batch;
 
 /* Meshes, materials (dt > 0) and options as for sim_create, HOST arrays,

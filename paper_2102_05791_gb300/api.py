@@ -144,7 +144,7 @@ class Simulator:
         return out
 
     def hvp_dot(self, x, a, v):
-        """(H v, v.(H v)) with the inner product formed as the CG loop forms p.Ap."""
+        """(H v, v.(H v)) with the inner product formed as the per-iteration CG loop forms p.Ap."""
         x, a = self._vec(x), self._elem(a)
         v = self._vec(v, self.vec_dtype, "v")
         out = self._empty(self.vec_dtype)

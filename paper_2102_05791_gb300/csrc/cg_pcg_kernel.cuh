@@ -13,7 +13,8 @@
 // Preconditioner.  z = D^-1 r + Z E^-1 Z^T r: inverse diagonal blocks plus a
 // Galerkin coarse correction over the rigid motions of 16-64 aggregates
 // (additive two-level Schwarz), symmetric positive definite and fixed during
-// a solve.  It cuts the iterations 2-7 times (the more the larger the mesh).
+// a solve (its coarse part in FP32 on FP64 handles too).  It cuts the iterations 2.5
+// to 7 times (the more the larger the mesh; 1.2 times at 256 triangles).
 //
 // Each CTA owns one part of the vertices.  Its x and r stay in registers, p
 // (with the halo's copy) and A p in shared memory.  Its edge slice is stored by
