@@ -8,7 +8,7 @@
 // the blocks kept in the team's shared memory: an iteration takes about 4.3 us
 // plus 6.4 ns per vertex on one CTA (24 us at 2,100 triangles when every
 // iteration gathered elements and corners through L2), and there are half as
-// many.  256 bodies of 200 to 8,000 triangles, 4 steps and back: 225 -> 64 ms;
+// many.  256 bodies of 200 to 8,000 triangles, 4 steps and back: 225 -> 60 ms;
 // 12 such bodies, 6 steps, on clusters: 230 -> 23 ms.
 // Spills cost much here (226 KB of shared memory leave the L1 28 KB): per-slot
 // addresses are looked up in the plan where they are used.  All passes are
